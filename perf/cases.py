@@ -285,6 +285,17 @@ def _network(case, seed):
     return n_in, n_out, H, p, m, v
 
 
+def _loading_head(p, n_out, H):
+    """The last layer as training leaves it: loadings around 10, preconditioner entries near diag(R + delta)^-1/2."""
+    p = p.copy()
+    w3 = p[p.size - n_out * (H + 1):p.size - n_out].reshape(n_out, H)
+    w3[0] *= 0.2
+    w3[1:] *= 0.02
+    p[-n_out] = 1.0
+    p[p.size - n_out + 1:] = -0.8
+    return p
+
+
 def _batch(case, seed, n_in, n_out):
     """Features and targets: correlated unit-scale columns, as covariance entries over their trace are."""
     g = _gen(seed, 1)
@@ -345,7 +356,7 @@ def prepare(case, seed):
     if kind == "loading":
         plan = _window_plan(case, seed)[2]
         n_in, n_out, H, p, _, _ = _network(case, seed)
-        p[-n_out] = 1.0   # an output bias in the range of the loadings (log10)
+        p = _loading_head(p, n_out, H)
         s = plan.sizes
         return dict(case=case, plan=plan, z=_windows(case, seed),
                     net=learned.LoadingMLP(n_in, n_out, H, capacity=4096, params=p),
@@ -639,7 +650,7 @@ def _exact_loading(case, seed):
     X = torch.cat([R.diagonal(dim1=1, dim2=2).real / tau[:, None], low.real, low.imag, an.real, an.imag,
                    tau.log10()[:, None], torch.full((G, 1), math.log10(K / W), device="cuda")], 1)
     n_in, n_out, H, p, _, _ = _network(case, seed)
-    p[-n_out] = 1.0
+    p = _loading_head(p, n_out, H)
     w = _layers(p, n_in, H, n_out)
     h = (X @ w["W1"].T + w["b1"]).clamp_min(0)
     h = (h @ w["W2"].T + w["b2"]).clamp_min(0)

@@ -8,7 +8,9 @@
 //   diag(R)/tau (W) | Re R_ij/tau, i > j row-major | Im R_ij/tau, same order |
 //   Re a/|a| (W) | Im a/|a| (W) | log10 tau | log10(K/W)      (W^2 + 2W + 2).
 // Weights are kept in FP32 (master, Adam) with a BF16 copy that the forward
-// and backward products read; all products accumulate in FP32.
+// and backward products read; all products accumulate in FP32.  Networks of
+// up to 256 hidden units and 64 outputs run in mlp_fused.cu; the layer by
+// layer products here serve the larger ones.
 #include <math.h>
 
 #include "common.cuh"
@@ -307,6 +309,7 @@ bs_status bs_mlp_forward(const bs_mlp *m, const float *X, int64_t batch, float *
     if (batch < 0 || batch > w->capacity) return set_error(BS_EINVAL, "batch exceeds the work buffers");
     if (batch == 0) return BS_OK;
     const cudaStream_t st = (cudaStream_t)stream;
+    if (bs::mlp_fused_applies(m) && batch <= INT32_MAX) return bs::launch_mlp_forward(m, X, (int)batch, Y, st);
     const int I = m->n_in, H = m->n_hidden, O = m->n_out, B = (int)batch;
     const __nv_bfloat16 *wb = (const __nv_bfloat16 *)m->weights_bf16;
     const float *b1 = m->master + (int64_t)H * I, *b2 = b1 + H + (int64_t)H * H, *b3 = b2 + H + (int64_t)O * H;
@@ -320,11 +323,22 @@ bs_status bs_mlp_forward(const bs_mlp *m, const float *X, int64_t batch, float *
 
 bs_status bs_mlp_train_step(bs_mlp *m, const float *X, const float *T, int64_t batch, const bs_mlp_work *w,
                             float lr, double *loss, bs_stream stream) {
-    if (bs_status s = bs_mlp_forward(m, X, batch, w->y, w, stream)) return s;
+    if (bs_status s = mlp_check(m)) return s;
+    const bool fused = bs::mlp_fused_applies(m) && batch >= 0 && batch <= INT32_MAX;
+    if (!fused) {
+        if (bs_status s = bs_mlp_forward(m, X, batch, w ? w->y : nullptr, w, stream)) return s;
+    } else {
+        if (!X || !w || !w->y || !w->z1 || !w->h1 || !w->z2 || !w->h2) return set_error(BS_EINVAL, "NULL buffer");
+        if (batch > w->capacity) return set_error(BS_EINVAL, "batch exceeds the work buffers");
+    }
     if (!T || !m->grad || !m->adam_m || !m->adam_v || !w->dy || !w->dh1 || !w->dh2)
         return set_error(BS_EINVAL, "NULL buffer");
     if (batch == 0) return BS_OK;
     const cudaStream_t st = (cudaStream_t)stream;
+    if (fused) {
+        if (lr > 0.f) m->step += 1;
+        return bs::launch_mlp_train(m, X, T, (int)batch, w, lr, m->step, loss, st);
+    }
     const int I = m->n_in, H = m->n_hidden, O = m->n_out, B = (int)batch;
     const int64_t P = bs_mlp_param_count(I, H, O);
     const __nv_bfloat16 *wb = (const __nv_bfloat16 *)m->weights_bf16;

@@ -45,7 +45,7 @@
 // word and the CTA stops after freeing its tensor memory.
 #include "beamspace_dev.cuh"
 #include "internal.h"
-#include "tma.cuh"
+#include "tcgen05.cuh"
 
 #include <algorithm>
 
@@ -96,19 +96,6 @@ struct TcArgs {
 
 // ---------------------------------------------------------------- PTX helpers
 
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
 // Shared-memory matrix descriptor, canonical K-major layout without swizzle:
 // 8-row x 16-byte core matrices, LBO = 128 bytes between core matrices
 // adjacent in K, SBO = 1024 bytes between 8-row groups.
@@ -126,11 +113,6 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t bdesc, u
         "r"(a), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
 // 32 consecutive 32-bit columns of this warp's lanes, two ranges, then wait.
 __device__ __forceinline__ void tmem_ld2x32(uint32_t a0, uint32_t a1, float (&r)[32], float (&s)[32]) {
     asm volatile(
@@ -164,21 +146,12 @@ __device__ __forceinline__ void tmem_st32(uint32_t a, const uint32_t (&v)[32]) {
         : "memory");
 }
 
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
-                 : "memory");
-}
-
 // Barrier of the four epilogue warps of vector pair g (named barriers 3, 4).
 __device__ __forceinline__ void group_bar(int g) {
     if (g == 0)
         asm volatile("bar.sync 3, 128;" ::: "memory");
     else
         asm volatile("bar.sync 4, 128;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ uint32_t half2_bits(float lo, float hi) {

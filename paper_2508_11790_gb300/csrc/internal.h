@@ -140,6 +140,13 @@ bs_status launch_window_cov_mma(const bs_plan *p, const void *ztr, const float *
 // dpre: optional diagonal preconditioner [c_elems] (woff-packed), NULL for none
 bs_status launch_mvdr_solve(const bs_plan *p, const double2 *R, float2 *c, int32_t *info,
                             cudaStream_t st, const float *dpre = nullptr);
+// the pairs of window size W <= 16, without and with a preconditioner, and of sizes W - 3 .. W (W = 20, 24, 28, 32)
+bs_status launch_solve_small(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
+                             const float *dpre, int refine, int f64);
+bs_status launch_solve_small_precond(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info,
+                                     cudaStream_t st, const float *dpre, int refine, int f64);
+bs_status launch_solve_wide(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
+                            const float *dpre, int refine, int f64);
 bs_status launch_apply(const bs_plan *p, const float2 *zte, const float2 *c, float2 *out,
                        cudaStream_t st);
 bs_status launch_cov_solve(const bs_plan *p, const void *ztr, const float *delta, double2 *R, float2 *c,

@@ -94,11 +94,17 @@ __device__ __forceinline__ float hw_sumf(unsigned mask, float x) {
     return x;
 }
 
+// Scratch of one group: its FP32 factor as rows of GW + 1 float2, or its FP64
+// factor as a packed lower triangle (entry (i, j) at i (i + 1) / 2 + j) --
+// the same number of bytes.
+template <int GW>
+constexpr int solve_scratch_bytes = GW * (GW + 1) * 8;
+
 // Whole solve in FP64 for one pair (escalation path), row `lane` of R given
 // in D.  Returns 0 or pivot+1.
 template <int GW = 16>
 static __device__ __forceinline__ int solve_f64_rows(unsigned mask, int lane, int W, double2 (&D)[GW], double2 a,
-                                     double2 (*Ld)[GW + 1], double2 &c_out) {
+                                                     double2 *Ld, double2 &c_out) {
     const bool row = lane < W;
 #pragma unroll
     for (int j = 0; j < GW; ++j)
@@ -129,7 +135,7 @@ static __device__ __forceinline__ int solve_f64_rows(unsigned mask, int lane, in
     if (fail) return fail;
 #pragma unroll
     for (int j = 0; j < GW; ++j)
-        if (row && j <= lane) Ld[lane][j] = D[j];
+        if (row && j <= lane) Ld[lane * (lane + 1) / 2 + j] = D[j];
     __syncwarp(mask);
     // one FP64 division per lane: GB300's FP64 pipe is narrow and a division
     // is a long sequence on it (two per step of each solve before)
@@ -156,7 +162,7 @@ static __device__ __forceinline__ int solve_f64_rows(unsigned mask, int lane, in
             const double2 vj = shfl2d<GW>(mask, mine, j);
             if (lane == j) v = vj;
             if (lane < j) {
-                const double2 t = dconjmul(Ld[j][lane], vj);
+                const double2 t = dconjmul(Ld[j * (j + 1) / 2 + lane], vj);
                 acc = make_double2(acc.x - t.x, acc.y - t.y);
             }
         }
@@ -188,7 +194,7 @@ __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned
 // 2^(ex_lane + ex_j), exactly.
 template <int GW = 16>
 static __device__ __noinline__ int solve_f64(unsigned mask, int lane, int W, const double2 *__restrict__ Rg, double2 a,
-                                double2 (*Ld)[GW + 1], double2 &c_out, int ex) {
+                                                double2 *Ld, double2 &c_out, int ex) {
     double2 D[GW];
     const bool row = lane < W;
 #pragma unroll
@@ -269,33 +275,48 @@ __device__ __forceinline__ float2 split_f64(double d) {
     return make_float2(__uint_as_float(hb), sign ? -lo : lo);
 }
 
-// Solve one pair of window size WT with the calling half-warp (lanes 0..15
-// of `mask`).  Rg: its W x W covariance in FP64 (row-major; global or shared
-// memory), read as FP32 (hi, lo) parts; a32/alo: the windowed steering
-// vector as hi / lo FP32 parts, a64 in FP64 (escalation).  scratch: [16][17]
-// double2 per half-warp.  Writes c[0..W) and *info.  Not inlined, so each
-// window size is compiled once per translation unit.
-template <int WT, int GW = 16>
-__device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const double2 *Rg,
-                                                     const float2 *__restrict__ a32g,
-                                                     const float2 *__restrict__ alog,
-                                                     const double2 *__restrict__ a64g, float2 *__restrict__ c,
-                                                     int32_t *__restrict__ info, double kappa_max, int refine,
-                                                     int allow_f64, double2 (*scratch)[GW + 1],
-                                                     const float *__restrict__ dg) {
-    const int ex = (dg && lane < WT) ? precond_exp(dg[lane]) : 0;   // this row's scaling exponent
-    int exj[WT];                                                     // every column's
+// Solve one pair of window size W <= WT with the calling group of GW lanes
+// (`lane` within it, `mask` its lanes of the warp).  Rg: its W x W covariance
+// in FP64 (row-major; global or shared memory), read as FP32 (hi, lo) parts;
+// a32/alo: the windowed steering vector as hi / lo FP32 parts, a64 in FP64
+// (escalation).  scratch: solve_scratch_bytes<GW> of shared memory.  Writes
+// c[0..W) and *info.
+//
+// W < WT: the matrix is padded with zero off-diagonal entries, R_00 on its
+// diagonal and the preconditioner entry of row 0, so the padded pivots equal
+// the pair's first (the pivot ratio that decides FP64 escalation is the
+// pair's); with zero steering entries there the padded solution entries are
+// exactly zero, and the first W entries are the W x W solve.
+// PRE: a preconditioner dg may be given (NULL for none).  LOCKSTEP: the whole
+// CTA calls this together and its warps meet at a barrier before every column
+// of the factorisation, so that they fetch its straight-line code once (a
+// pair past the end is solved for an `active` = false group that stores
+// nothing).
+template <int WT, int GW, bool PRE, bool LOCKSTEP = false>
+__device__ __forceinline__ void solve_pair_core(unsigned mask, int lane, int W, const double2 *Rg,
+                                                const float2 *__restrict__ a32g, const float2 *__restrict__ alog,
+                                                const double2 *__restrict__ a64g, float2 *__restrict__ c,
+                                                int32_t *__restrict__ info, double kappa_max, int refine,
+                                                int allow_f64, void *scratch, const float *__restrict__ dg,
+                                                bool active = true) {
+    const bool row = lane < W;
+    // this row's scaling exponent and every column's
+    const int ex = (PRE && dg && lane < WT) ? precond_exp(dg[row ? lane : 0]) : 0;
+    int exj[PRE ? WT : 1];
+    if constexpr (PRE) {
 #pragma unroll
-    for (int j = 0; j < WT; ++j) exj[j] = __shfl_sync(mask, ex, j, GW);
+        for (int j = 0; j < WT; ++j) exj[j] = __shfl_sync(mask, ex, j, GW);
+    }
     auto rows = [&](int j) -> float4 {
-        const double2 r = Rg[lane * WT + j];
+        double2 r = make_double2(0.0, 0.0);
+        if (row && j < W) r = Rg[lane * W + j];
+        else if (lane == j) r = Rg[0];
         const float2 x = split_f64(r.x), y = split_f64(r.y);
-        const float s = pow2f(ex + exj[j]);   // exact: a power of two
+        if constexpr (!PRE) return make_float4(x.x, y.x, x.y, y.y);
+        const float s = pow2f(ex + exj[PRE ? j : 0]);   // exact: a power of two
         return make_float4(x.x * s, y.x * s, x.y * s, y.y * s);
     };
-    float2(*Lsf)[GW + 1] = reinterpret_cast<float2(*)[GW + 1]>(&scratch[0][0]);
-    constexpr int W = WT;
-    const bool row = lane < W;
+    float2(*Lsf)[GW + 1] = static_cast<float2(*)[GW + 1]>(scratch);
 
     // Up to kKeepRow entries the lane's split row stays in registers for the
     // refinement residual (else it is read and split again there).
@@ -307,7 +328,7 @@ __device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const d
 #pragma unroll
     for (int j = 0; j < WT; ++j) {
         float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row) r = rows(j);
+        if (lane < WT) r = rows(j);
         finite = finite && isfinite(r.x) && isfinite(r.y);
         A[j] = make_float2(r.x, r.y);
         if constexpr (WT <= kKeepRow) Rrow[j] = r;
@@ -316,7 +337,8 @@ __device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const d
     const float2 ah = row ? cscale(a32g[lane], sa) : make_float2(0.f, 0.f);
     const float2 al = row ? cscale(alog[lane], sa) : make_float2(0.f, 0.f);
     finite = finite && isfinite(ah.x) && isfinite(ah.y);
-    if (!__all_sync(mask, finite)) {
+    finite = __all_sync(mask, finite);
+    if (!LOCKSTEP && !finite) {
         if (row) c[lane] = make_float2(nanf(""), nanf(""));
         if (lane == 0) *info = -1;
         return;
@@ -327,6 +349,7 @@ __device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const d
     float diag = 1.f, dmax = 0.f, dmin = INFINITY;
 #pragma unroll
     for (int k = 0; k < WT; ++k) {
+        if constexpr (LOCKSTEP) __syncthreads();
         const float dkk = __shfl_sync(mask, A[k].x, k, GW);
         if (!(dkk > 0.f) && fail == 0) fail = k + 1;
         const float inv = rsqrtf(dkk > 0.f ? dkk : 1.f);   // the refinement step absorbs its last-bit error
@@ -341,12 +364,20 @@ __device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const d
             if (lane >= j) A[j] = csub(A[j], cmulc(A[k], ljk));
         }
     }
+    if constexpr (LOCKSTEP) {   // no barrier below
+        if (!active) return;
+        if (!finite) {
+            if (row) c[lane] = make_float2(nanf(""), nanf(""));
+            if (lane == 0) *info = -1;
+            return;
+        }
+    }
     const float ratio = dmax / dmin;
     const bool escalate = allow_f64 && (fail != 0 || ratio * ratio > (float)kappa_max);
     if (!escalate && fail == 0) {
 #pragma unroll
         for (int j = 0; j < WT; ++j)
-            if (row && j <= lane) Lsf[lane][j] = A[j];
+            if (lane < WT && j <= lane) Lsf[lane][j] = A[j];
         __syncwarp(mask);
         // 2. solve in FP32
         float2 v = chol_solve_f32<WT, GW>(mask, lane, A, diag, Lsf, ah);
@@ -372,7 +403,7 @@ __device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const d
         return;
     }
     // FP64 path
-    double2(*Ldd)[GW + 1] = scratch;
+    double2 *Ldd = static_cast<double2 *>(scratch);
     __syncwarp(mask);
     double2 cd;
     const double2 a64 = row ? a64g[lane] : make_double2(0.0, 0.0);
@@ -386,18 +417,18 @@ __device__ __forceinline__ void solve_pair_body(unsigned mask, int lane, const d
     if (lane == 0) *info = -2;
 }
 
-// The same solve as a separate function per window size (the fused and
-// whole-warp kernels call it: one copy of the body per W and translation
-// unit, and their own registers stay free of it).
-template <int WT, int GW = 16>
+// The same solve as a separate function per window size (the fused kernel
+// calls it: one copy of the body per W and translation unit, and its own
+// registers stay free of it).
+template <int WT>
 static __device__ __noinline__ void solve_pair_fixed(unsigned mask, int lane, const double2 *Rg,
                                                      const float2 *__restrict__ a32g,
                                                      const float2 *__restrict__ alog,
                                                      const double2 *__restrict__ a64g, float2 *__restrict__ c,
                                                      int32_t *__restrict__ info, double kappa_max, int refine,
-                                                     int allow_f64, double2 (*scratch)[GW + 1],
-                                                     const float *__restrict__ dg) {
-    solve_pair_body<WT, GW>(mask, lane, Rg, a32g, alog, a64g, c, info, kappa_max, refine, allow_f64, scratch, dg);
+                                                     int allow_f64, void *scratch, const float *__restrict__ dg) {
+    solve_pair_core<WT, 16, true>(mask, lane, WT, Rg, a32g, alog, a64g, c, info, kappa_max, refine, allow_f64, scratch,
+                                  dg);
 }
 
 // R stored as FP64 (global or shared memory); dispatches on W to the solve
@@ -406,7 +437,7 @@ __device__ __forceinline__ void solve_pair(unsigned mask, int lane, int W, const
                                            const float2 *__restrict__ a32g, const float2 *__restrict__ alog,
                                            const double2 *__restrict__ a64g, float2 *__restrict__ c,
                                            int32_t *__restrict__ info, double kappa_max, int refine,
-                                           int allow_f64, double2 (*scratch)[WMAX + 1],
+                                           int allow_f64, void *scratch,
                                            const float *__restrict__ dg = nullptr) {
 #define BS_SOLVE_CASE(n) \
     case n: solve_pair_fixed<n>(mask, lane, Rg, a32g, alog, a64g, c, info, kappa_max, refine, allow_f64, scratch, dg); break;

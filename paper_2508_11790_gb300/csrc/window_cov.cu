@@ -180,6 +180,170 @@ __global__ void __launch_bounds__(COV_THREADS)
     }
 }
 
+// Plans with windows above 16 beams: one CTA per pair with 4 x 4 tiles.  The
+// 3 x 3 tiles of window_cov_kernel left 62 of 128 threads idle at W = 32 (66
+// tiles, one slice) and tested every entry against W; here 36 tiles fill 108
+// threads in three slices, rows are staged at a pitch of a multiple of four
+// with zero entries past W, and a thread reads its eight entries as four
+// 16-byte loads per 64 FMA.  Bound by issue (FMA and their loads) and by the
+// FP64 conversions of R: 2560 pairs of W = 32, K = 128 take 91 us (113 with
+// the 3 x 3 tiles).
+constexpr int CW_ELEMS = 1024;   // padded window entries per staging buffer
+
+// Position of entry w in a staged row: pairs of entries (16 bytes in FP32) 8
+// and up swap with their neighbour, so that the first halves of eight tiles'
+// entries (32 bytes apart) lie in distinct banks.
+__device__ __forceinline__ int cw_pos(int w) { return w ^ ((w >> 3) & 2); }
+
+// The four staged entries of tile b of the row at o.
+template <int PREC>
+__device__ __forceinline__ void widen4(const void *stage, int o, int b, float inv_sc, float2 (&z)[4]) {
+    const int q = o + 4 * b;
+    if constexpr (PREC == BS_PREC_FP32) {
+        const float4 *p = reinterpret_cast<const float4 *>(reinterpret_cast<const float2 *>(stage) + q);
+        const int sw = (b >> 2) & 1;
+        const float4 u = p[sw], v = p[sw ^ 1];
+        z[0] = make_float2(u.x, u.y);
+        z[1] = make_float2(u.z, u.w);
+        z[2] = make_float2(v.x, v.y);
+        z[3] = make_float2(v.z, v.w);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z[k] = widen<PREC>(stage, o + cw_pos(4 * b + k), inv_sc);
+    }
+}
+
+template <int PREC>
+__global__ void __launch_bounds__(COV_THREADS, 4)
+    window_cov_wide_kernel(const void *__restrict__ z, const int64_t *__restrict__ ztr_off,
+                           const int32_t *__restrict__ Wg, const int32_t *__restrict__ Kg,
+                           const int64_t *__restrict__ roff, const float *__restrict__ delta_pair, DF delta,
+                           float inv_sc, double2 *__restrict__ R) {
+    constexpr int ES = (PREC == BS_PREC_FP32) ? 8 : 4;   // bytes per stored element
+    __shared__ __align__(16) union {
+        unsigned char stage[2][CW_ELEMS * ES];
+        float red[4][16][COV_THREADS];   // the slices' sums, after the last chunk
+    } sm;
+    const int64_t g = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int W = Wg[g], K = Kg[g];
+    const int nb = (W + 3) / 4, Wp = 4 * nb;
+    const int ntile = nb * (nb + 1) / 2;
+    const int H = COV_THREADS / ntile;
+    const int tile = tid % ntile, h = tid / ntile;
+    const bool active = h < H;
+    int bi = 0, bj = tile;
+    while (bj > bi) { bj -= bi + 1; ++bi; }
+    const int kc = CW_ELEMS / Wp;   // vectors per chunk
+    const unsigned char *zg = reinterpret_cast<const unsigned char *>(z) + ztr_off[g] * ES;
+
+    for (int b = 0; b < 2; ++b)   // the entries past W, never written again
+        for (int q = tid; q < kc * (Wp - W); q += COV_THREADS) {
+            unsigned char *d = &sm.stage[b][((q / (Wp - W)) * Wp + cw_pos(W + q % (Wp - W))) * ES];
+            if constexpr (ES == 8) *reinterpret_cast<float2 *>(d) = make_float2(0.f, 0.f);
+            else *reinterpret_cast<uint32_t *>(d) = 0;
+        }
+    auto issue = [&](int k0, int buf) {
+        const int n = min(kc, K - k0);
+        if (lane < W)
+            for (int v = warp; v < n; v += COV_THREADS / 32)
+                cp_async<ES>(&sm.stage[buf][(v * Wp + cw_pos(lane)) * ES], zg + ((int64_t)(k0 + v) * W + lane) * ES);
+        cp_async_commit();
+    };
+
+    float ar[4][4], ai[4][4], hr[4][4], lr[4][4], hi[4][4], li[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ar[r][q] = ai[r][q] = hr[r][q] = lr[r][q] = hi[r][q] = li[r][q] = 0.f;
+    auto fold = [&]() {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                df_add(hr[r][q], lr[r][q], ar[r][q]);
+                df_add(hi[r][q], li[r][q], ai[r][q]);
+                ar[r][q] = ai[r][q] = 0.f;
+            }
+    };
+    int cnt = 0, buf = 0;
+    issue(0, 0);
+    for (int k0 = 0; k0 < K; k0 += kc, buf ^= 1) {
+        const int n = min(kc, K - k0);
+        if (k0 + kc < K) {
+            issue(k0 + kc, buf ^ 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
+        if (active) {
+            for (int v = h; v < n; v += H) {
+                float2 zi[4], zj[4];
+                widen4<PREC>(sm.stage[buf], v * Wp, bi, inv_sc, zi);
+                widen4<PREC>(sm.stage[buf], v * Wp, bj, inv_sc, zj);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {   // z_i conj(z_j)
+                        ar[r][q] = fmaf(zi[r].x, zj[q].x, fmaf(zi[r].y, zj[q].y, ar[r][q]));
+                        ai[r][q] = fmaf(zi[r].y, zj[q].x, fmaf(-zi[r].x, zj[q].y, ai[r][q]));
+                    }
+                if (++cnt == 16) {
+                    fold();
+                    cnt = 0;
+                }
+            }
+        }
+        __syncthreads();   // this stage is reloaded two chunks later
+    }
+    fold();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            sm.red[0][4 * r + q][tid] = hr[r][q];
+            sm.red[1][4 * r + q][tid] = lr[r][q];
+            sm.red[2][4 * r + q][tid] = hi[r][q];
+            sm.red[3][4 * r + q][tid] = li[r][q];
+        }
+    __syncthreads();
+
+    // 1/K, the loading and R in double-float; FP64 only for the stored values
+    const float Kf = (float)K;
+    const float qk = 1.f / Kf;
+    const DF invK = df_norm(qk, fmaf(-qk, Kf, 1.f) / Kf);
+    const DF dl = delta_pair ? DF{delta_pair[g], 0.f} : delta;
+    double2 *Rg = R + roff[g];
+    // lower-triangle entries in order, every lane busy: the FP64 conversions
+    // (a narrow pipe) were a third of the kernel with a row per warp
+    const int E = W * (W + 1) / 2;
+    for (int e = tid; e < E; e += COV_THREADS) {
+        int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+        i += (i + 1) * (i + 2) / 2 <= e;   // the rounded root may be one off
+        i -= i * (i + 1) / 2 > e;
+        const int j = e - i * (i + 1) / 2;
+        const int b = (i / 4) * (i / 4 + 1) / 2 + j / 4;
+        const int ee = 4 * (i % 4) + (j % 4);
+        float sh = 0.f, sl = 0.f, th = 0.f, tl = 0.f;
+        for (int hh = 0; hh < H; ++hh) {
+            const int o = hh * ntile + b;
+            df_add(sh, sl, sm.red[0][ee][o]);
+            sl += sm.red[1][ee][o];
+            df_add(th, tl, sm.red[2][ee][o]);
+            tl += sm.red[3][ee][o];
+        }
+        const DF re = df_mul(df_norm(sh, sl), invK);
+        if (i == j) {
+            Rg[i * W + i] = make_double2(df_to_double(df_add(re, dl)), 0.0);
+        } else {
+            const double rd = df_to_double(re), id = df_to_double(df_mul(df_norm(th, tl), invK));
+            Rg[i * W + j] = make_double2(rd, id);
+            Rg[j * W + i] = make_double2(rd, __longlong_as_double(__double_as_longlong(id) ^ (1ll << 63)));
+        }
+    }
+}
+
 // Short window streams (K <= 128): one warp per pair, four pairs per CTA.
 // The warp stages chunks of 64 vectors of its pair with coalesced loads;
 // lane l owns entries e = l + 32 k (k < ceil(E / 32) <= 5) of the lower
@@ -375,8 +539,8 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
                                                                    p->d_Kg, p->d_roff, delta, (float)p->cfg.delta, R);
         return check_launch("plain covariance launch");
     }
-    // windows above 16 beams: the CTA-per-pair kernel (its 3 x 3 tiles cover
-    // any W; 16-bit windows are widened to FP32 as they are staged)
+    // windows above 16 beams: a CTA per pair with 4 x 4 tiles, which cover any
+    // W (16-bit windows are widened to FP32 as they are read)
     const bool wide = p->Wmax > WMAX_COV;
     if (wide && p->Wmax > 32) return set_error(BS_EUNSUPPORTED, "W > 32");
     const int tv = p->tune_cov;   // a variant chosen by bs_autotune_pass, where it applies
@@ -386,6 +550,15 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
     const float inv_sc = 1.0f / p->cfg.store_scale;
     // warp per pair: short streams over enough pairs to fill the GPU by warps
     if (window_cov_uses_warp(p)) return launch_window_cov_warp(p, ztr, delta, R, st, 0, p->pairs, nullptr);
+    if (wide) {
+        const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_wide_kernel<BS_PREC_FP32>
+                            : p->cfg.precision == BS_PREC_FP16 ? window_cov_wide_kernel<BS_PREC_FP16>
+                                                               : window_cov_wide_kernel<BS_PREC_BF16>;
+        kernel<<<G, COV_THREADS, 0, st>>>(ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta,
+                                          df_from_double(p->cfg.delta),
+                                          p->cfg.precision == BS_PREC_FP32 ? 1.0f : inv_sc, R);
+        return check_launch("covariance (wide windows) launch");
+    }
     switch (p->cfg.precision) {
         case BS_PREC_FP32:
             window_cov_kernel<BS_PREC_FP32><<<G, COV_THREADS, 0, st>>>(

@@ -3,24 +3,133 @@
 // OverallWindow read as S_h (x) S_v, Eq. ApplyWindow).
 //
 // Elements n = n_x Nz + n_z, beams m = m_x Mz + m_z, window entries
-// w = w_x Wz + w_z.  One warp per (record, bin) vector, several per CTA: the
-// vector's N = Nx Nz elements are staged in the warp's shared memory; the
-// vertical DFT (Mz points of Nz, D_v) runs as direct sums into Mz rows of
-// Mx points, zero beyond Nx, and the horizontal one (Mx points, D_h^T) as a
-// radix-2 Stockham FFT along every row (log2 Mx passes, two buffers,
-// twiddles from an exact per-CTA table), leaving all M = Mx Mz beams with
-// row m_z holding m_x in natural order.  The window gather then takes the
-// plan's flat (target, entry) list a lane per entry and writes every
-// target's Wx x Wz window to the packed window arrays with the conventions
-// of the linear-array kernels.  Only warp barriers inside the vector loop.
-// Planar plans are limited to N <= 1024 and M <= 2048 (the paper's array
-// is 4 x 32).
+// w = w_x Wz + w_z.  Planar plans are limited to N <= 1024 and M <= 2048 (the
+// paper's array is 4 x 32).
+//
+// beamspace2d_fft_kernel: a CTA takes 4096 / M consecutive vectors.  A thread
+// loads one column of Nz elements straight from memory, takes its Mz-point
+// DFT in registers and writes Mz rows of the shared buffer; all 4096 / Mx rows
+// then go through the Mx-point Stockham passes of the linear kernels (zero
+// past Nx).  The vectors of a subband share their targets' windows, so a
+// thread decodes a (target, entry) once and stores it for all of them.  Bound
+// by the window stores: 20 targets of 4 x 8 beams write 5 KB per 1 KB vector.
+// 24 576 vectors of 4 x 32 elements, 8 x 64 beams: 37 us (22 us at the copy
+// bandwidth; 195 us with the general kernel).
+//
+// beamspace2d_kernel: any other shape; one warp per vector (radix-2 passes in
+// shared memory, direct vertical sums, every entry decoded per vector).
 #include "beamspace_dev.cuh"
 #include "internal.h"
 
 #include <algorithm>
 
 namespace bs {
+
+// Targets of the current subband: window-array base of its first vector, window
+// starts, and how many of its vectors store.
+struct __align__(16) Tgt2d {
+    long long base;
+    int sxz;   // start_x | start_z << 16
+    int wn;    // W | Wz << 8 | stores << 16
+};
+
+constexpr int kPts2d = 4096;   // points per CTA
+
+template <int MZ>
+__device__ __forceinline__ void column_dft(const float2 *__restrict__ y, int Nz, bool valid, float2 *b, int pitch) {
+    float2 a[MZ];
+#pragma unroll
+    for (int k = 0; k < MZ; ++k) a[k] = (valid && k < Nz) ? __ldg(y + k) : make_float2(0.f, 0.f);
+    RegDFT<MZ>::run(a);
+#pragma unroll
+    for (int k = 0; k < MZ; ++k) b[k * pitch] = a[k];
+}
+
+template <int MX>
+__global__ void __launch_bounds__(256, 4)
+    beamspace2d_fft_kernel(const float2 *__restrict__ y, int Nx, int Nz, int Mz, float scale, int prec, GatherArgs ga,
+                           const int32_t *__restrict__ start_z, const int32_t *__restrict__ Wz,
+                           const int32_t *__restrict__ glist, int sumW, const float2 *__restrict__ tw) {
+    using RP = Radix<MX>;
+    constexpr int rows = kPts2d / MX, pl = padded_len(MX), nthr = 256;
+    __shared__ float2 b[rows * pl];
+    __shared__ float2 twx[MX];
+    __shared__ Tgt2d tgt[kTabT];
+    const int tid = threadIdx.x;
+    const int N = Nx * Nz, V = rows / Mz;   // vectors of this CTA
+    const int64_t vid0 = (int64_t)blockIdx.x * V;
+    for (int k = tid; k < MX; k += nthr) twx[k] = __ldg(&tw[k * Mz]);
+    for (int c = tid; c < V * Nx; c += nthr) {   // columns (v, n_x)
+        const int v = c / Nx, nx = c - v * Nx;
+        const bool valid = vid0 + v < ga.nvec;
+        const float2 *col = y + (valid ? (vid0 + v) * N + nx * Nz : 0);
+        float2 *d = b + v * Mz * pl + padrow(nx);
+        switch (Mz) {
+            case 1: column_dft<1>(col, Nz, valid, d, pl); break;
+            case 2: column_dft<2>(col, Nz, valid, d, pl); break;
+            case 4: column_dft<4>(col, Nz, valid, d, pl); break;
+            case 8: column_dft<8>(col, Nz, valid, d, pl); break;
+            default: column_dft<16>(col, Nz, valid, d, pl); break;
+        }
+    }
+    __syncthreads();
+    auto twl = [&](int k) -> float2 { return twx[k]; };
+    auto cload = [&](int r, int t) -> float2 { return t < Nx ? b[r * pl + padrow(t)] : make_float2(0.f, 0.f); };
+    auto sload = [&](int r, int t) -> float2 { return b[r * pl + padrow(t)]; };
+    auto sstore = [&](int r, int t, float2 v) { b[r * pl + padrow(t)] = v; };
+    stockham_pass_tw<MX, RP::r0, 1, rows, nthr, false, true>(tid, twl, cload, sstore);
+    __syncthreads();
+    if constexpr (RP::npass >= 2) {
+        stockham_pass_tw<MX, RP::r1, RP::r0, rows, nthr, false, true>(tid, twl, sload, sstore);
+        __syncthreads();
+    }
+    if constexpr (RP::npass >= 3) {
+        stockham_pass_tw<MX, RP::r2, RP::r0 * RP::r1, rows, nthr, false, true>(tid, twl, sload, sstore);
+        __syncthreads();
+    }
+
+    // window stores, the vectors of one subband at a time
+    const int Bv = min(V, 1 << ga.log2B);
+    for (int g0 = 0; g0 < V && vid0 + g0 < ga.nvec; g0 += Bv) {
+        const int64_t vec = ga.vbase + vid0 + g0;
+        const int p = (int)(vec >> ga.log2F);
+        const int q = (int)(vec & ((1 << ga.log2F) - 1));
+        const int s = q >> ga.log2B, i = q & ((1 << ga.log2B) - 1);
+        const bool train = p < ga.P_train;
+        const int v0 = train ? (p << ga.log2B) + i : ((p - ga.P_train) << ga.log2B) + i;
+        for (int t = tid; t < ga.T; t += nthr) {
+            const int64_t g = (int64_t)t * ga.L + s;
+            const int W = __ldg(&ga.Wg[g]);
+            const int n = train ? max(0, min(Bv, __ldg(&ga.Kg[g]) - v0)) : Bv;
+            Tgt2d e;
+            e.base = __ldg(train ? &ga.ztr_off[g] : &ga.zte_off[g]) + (long long)v0 * W;
+            e.sxz = __ldg(&ga.start[g]) | (__ldg(&start_z[g]) << 16);
+            e.wn = W | (__ldg(&Wz[t]) << 8) | (n << 16);
+            tgt[t] = e;
+        }
+        __syncthreads();
+        const float2 *bg = b + g0 * Mz * pl;
+        for (int e = tid; e < sumW; e += nthr) {
+            const int packed = __ldg(&glist[e]);
+            const int w = packed & 255;
+            const Tgt2d te = tgt[packed >> 8];
+            const int W = te.wn & 255, wz = (te.wn >> 8) & 255, n = te.wn >> 16;
+            const int wx = w / wz;
+            const int mx = ((te.sxz & 0xFFFF) + wx) & (MX - 1), mz = ((te.sxz >> 16) + w - wx * wz) & (Mz - 1);
+            const float2 *src = bg + mz * pl + padrow(mx);
+            const int64_t o = te.base + w;
+            auto all = [&](auto put) {
+#pragma unroll 4
+                for (int v = 0; v < n; ++v) put(o + (int64_t)v * W, cscale(src[v * Mz * pl], scale));
+            };
+            if (!train) all([&](int64_t k, float2 v) { ga.zte[k] = v; });
+            else if (prec == BS_PREC_FP32) all([&](int64_t k, float2 v) { store_train<BS_PREC_FP32>(ga.ztr, k, v, 1.f); });
+            else if (prec == BS_PREC_FP16) all([&](int64_t k, float2 v) { store_train<BS_PREC_FP16>(ga.ztr, k, v, ga.store_scale); });
+            else all([&](int64_t k, float2 v) { store_train<BS_PREC_BF16>(ga.ztr, k, v, ga.store_scale); });
+        }
+        __syncthreads();   // the entries are rewritten for the next subband
+    }
+}
 
 __global__ void __launch_bounds__(128)
     beamspace2d_kernel(const float2 *__restrict__ y, int Nx, int Nz, int Mx, int Mz, float scale, int prec,
@@ -107,9 +216,34 @@ __global__ void __launch_bounds__(128)
     }
 }
 
+template <int MX>
+static bs_status launch_2d_fft(const bs_plan *p, const float2 *xc, const GatherArgs &ga, cudaStream_t st) {
+    const int V = kPts2d / (MX * p->Mz);
+    const int64_t blocks = (ga.nvec + V - 1) / V;
+    if (blocks > 0x7FFFFFFF) return set_error(BS_EUNSUPPORTED, "too many vectors");
+    beamspace2d_fft_kernel<MX><<<(unsigned)blocks, 256, 0, st>>>(
+        xc, p->Nx, p->Nz, p->Mz, 1.0f / sqrtf((float)(MX * p->Mz)), p->cfg.precision, ga, p->d_start_z, p->d_Wz,
+        p->d_glist, p->sumW, p->d_twM);
+    return check_launch("planar beamspace launch");
+}
+
 bs_status launch_beamspace2d(const bs_plan *p, const float2 *xc, const GatherArgs &ga, cudaStream_t st) {
     const int Nx = p->Nx, Nz = p->Nz, Mx = p->Mx, Mz = p->Mz;
     if (ga.nvec == 0) return BS_OK;
+    // rows of 8 to 1024 beams (Stockham radices), columns of up to 16 (in
+    // registers), 2 to 32 vectors per CTA, targets within the entry table
+    if (Mx >= 8 && Mx <= 1024 && Mz <= 16 && Mx * Mz >= 128 && p->cfg.T <= kTabT) {
+        switch (Mx) {
+            case 8: return launch_2d_fft<8>(p, xc, ga, st);
+            case 16: return launch_2d_fft<16>(p, xc, ga, st);
+            case 32: return launch_2d_fft<32>(p, xc, ga, st);
+            case 64: return launch_2d_fft<64>(p, xc, ga, st);
+            case 128: return launch_2d_fft<128>(p, xc, ga, st);
+            case 256: return launch_2d_fft<256>(p, xc, ga, st);
+            case 512: return launch_2d_fft<512>(p, xc, ga, st);
+            default: return launch_2d_fft<1024>(p, xc, ga, st);
+        }
+    }
     const size_t per_warp = ((size_t)Nx * Nz + 2 * (size_t)Mx * Mz) * sizeof(float2);
     const size_t tables = ((size_t)Mx / 2 + Mz) * sizeof(float2);
     // up to 4 vectors (warps) per CTA while their buffers stay within 48 KB

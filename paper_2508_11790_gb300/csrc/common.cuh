@@ -92,22 +92,22 @@ struct Radix {
 // products of at most three table entries, which keeps their error within
 // a few FP32 ulps while cutting the table loads per butterfly from R-1 to
 // at most 4 (the loads of a warp hit scattered table lines).
-template <int R>
-__device__ __forceinline__ void twiddle_powers(const float2 *__restrict__ tw, int e, float2 (&w)[R]) {
+template <int R, class Tw>
+__device__ __forceinline__ void twiddle_powers(Tw tw, int e, float2 (&w)[R]) {
     w[0] = make_float2(1.f, 0.f);
-    w[1] = __ldg(&tw[e]);
+    w[1] = tw(e);
     if constexpr (R >= 4) {
         w[2] = cmul(w[1], w[1]);
         w[3] = cmul(w[2], w[1]);
     }
     if constexpr (R >= 8) {
-        w[4] = __ldg(&tw[4 * e]);
+        w[4] = tw(4 * e);
 #pragma unroll
         for (int r = 5; r < 8; ++r) w[r] = cmul(w[4], w[r - 4]);
     }
     if constexpr (R >= 16) {
-        w[8] = __ldg(&tw[8 * e]);
-        w[12] = __ldg(&tw[12 * e]);
+        w[8] = tw(8 * e);
+        w[12] = tw(12 * e);
 #pragma unroll
         for (int r = 9; r < 12; ++r) w[r] = cmul(w[8], w[r - 8]);
 #pragma unroll
@@ -125,11 +125,10 @@ __device__ __forceinline__ void twiddle_powers(const float2 *__restrict__ tw, in
 // kSyncMid the pass reads everything into registers, synchronises the CTA
 // and then writes (in-place passes through shared memory).
 // kColFast: butterfly id -> (column = id % ncols) else (column = id / (n/R)).
-// tw[k] = e^{-2 pi i k / n}, k < n.
-template <int n, int R, int Ns, int ncols, int nthr, bool kColFast, bool kSyncMid,
+// tw(k) = e^{-2 pi i k / n}, k < n.
+template <int n, int R, int Ns, int ncols, int nthr, bool kColFast, bool kSyncMid, class Tw,
           class Load, class Store>
-__device__ __forceinline__ void stockham_pass(int tid, const float2 *__restrict__ tw, Load load,
-                                              Store store) {
+__device__ __forceinline__ void stockham_pass_tw(int tid, Tw tw, Load load, Store store) {
     constexpr int nb = ncols * (n / R);
     static_assert(nb % nthr == 0, "butterflies must divide evenly over threads");
     constexpr int bpt = nb / nthr;
@@ -143,7 +142,7 @@ __device__ __forceinline__ void stockham_pass(int tid, const float2 *__restrict_
         for (int r = 0; r < R; ++r) v[b][r] = load(c, j + r * (n / R));
         if (Ns > 1) {
             float2 w[R];
-            twiddle_powers<R>(tw, (j % Ns) * (n / (Ns * R)), w);
+            twiddle_powers(tw, (j % Ns) * (n / (Ns * R)), w);
 #pragma unroll
             for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
         }
@@ -160,6 +159,13 @@ __device__ __forceinline__ void stockham_pass(int tid, const float2 *__restrict_
 #pragma unroll
         for (int r = 0; r < R; ++r) store(c, base + r * Ns, v[b][r]);
     }
+}
+
+// The pass with the twiddles in global memory, tw[k] = e^{-2 pi i k / n}.
+template <int n, int R, int Ns, int ncols, int nthr, bool kColFast, bool kSyncMid, class Load, class Store>
+__device__ __forceinline__ void stockham_pass(int tid, const float2 *__restrict__ tw, Load load, Store store) {
+    stockham_pass_tw<n, R, Ns, ncols, nthr, kColFast, kSyncMid>(
+        tid, [tw](int k) { return __ldg(&tw[k]); }, load, store);
 }
 
 // Double-float values (h + l, |l| <= ulp(h)/2): GB300's FP64 pipe is

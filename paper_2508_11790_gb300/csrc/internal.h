@@ -166,8 +166,6 @@ int beamspace_vectors_per_cta(int M);
 // the tensor-core beamspace kernel serves this plan (beamspace_tc.cu)
 bool beamspace_tc_applies(const bs_plan *p);
 bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStream_t st);
-// orthonormal F-point DFT of nvec contiguous rows of F elements (F-point twiddle table)
-bs_status launch_fft_rows(const bs_plan *p, const float2 *y, int64_t nvec, float2 *yb, cudaStream_t st);
 bs_status launch_range_doppler(const bs_plan *p, const float2 *out, const float2 *pulse, float2 *work, float *map,
                                cudaStream_t st);
 bs_status launch_cfar(const bs_plan *p, const float *map, float threshold_db, float *floor, int32_t *count,

@@ -681,7 +681,7 @@ MlpArgs slab_args(const bs_mlp *m, const float *X, int batch, float *Y) {
 
 }  // namespace
 
-bool mlp_fused_applies(const bs_mlp *m) { return m->n_hidden <= 256 && m->n_out <= OMAX; }
+bool mlp_fused_applies(const bs_mlp *m) { return m->n_hidden <= 256 && m->n_out <= OMAX && m->n_in <= 65536; }
 
 bs_status launch_mlp_forward(const bs_mlp *m, const float *X, int batch, float *Y, cudaStream_t st) {
     const MlpArgs a = slab_args(m, X, batch, Y);
@@ -732,7 +732,6 @@ bs_status launch_mlp_train(const bs_mlp *m, const float *X, const float *T, int 
     g.eps = 1e-8f;
     g.bc1 = 1.f - powf(0.9f, (float)step);
     g.bc2 = 1.f - powf(0.999f, (float)step);
-    if (ntiles > 65535) return set_error(BS_EUNSUPPORTED, "too many input features");
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(S, ntiles);
     cfg.blockDim = dim3(256);

@@ -15,37 +15,105 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "solve_dev.cuh"
 
 namespace bs {
 
 // ----------------------------------------------------------------- features
-__global__ void features_kernel(const double2 *__restrict__ R, const int64_t *__restrict__ roff,
-                                const int32_t *__restrict__ Wg, const int32_t *__restrict__ Kg,
-                                const int64_t *__restrict__ woff, const double2 *__restrict__ at64,
-                                int64_t pairs, int nfeat, float *__restrict__ X) {
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= pairs) return;
-    const int W = Wg[g];
-    const double2 *Rg = R + roff[g];
-    const double2 *a = at64 + woff[g];
-    float *x = X + g * nfeat;
-    double tr = 0.0;
-    for (int i = 0; i < W; ++i) tr += Rg[i * W + i].x;
-    const double tau = tr / W;
-    const double itau = 1.0 / tau;
-    int o = 0;
-    for (int i = 0; i < W; ++i) x[o++] = (float)(Rg[i * W + i].x * itau);
-    for (int i = 1; i < W; ++i)
-        for (int j = 0; j < i; ++j) x[o++] = (float)(Rg[i * W + j].x * itau);
-    for (int i = 1; i < W; ++i)
-        for (int j = 0; j < i; ++j) x[o++] = (float)(Rg[i * W + j].y * itau);
-    double na = 0.0;
-    for (int i = 0; i < W; ++i) na += a[i].x * a[i].x + a[i].y * a[i].y;
-    const double ina = 1.0 / sqrt(na);
-    for (int i = 0; i < W; ++i) x[o++] = (float)(a[i].x * ina);
-    for (int i = 0; i < W; ++i) x[o++] = (float)(a[i].y * ina);
-    x[o++] = (float)log10(tau);
-    x[o++] = (float)log10((double)Kg[g] / (double)W);
+// FEAT_PAIRS pairs per CTA: first a thread per pair forms the pair's scalars,
+// then a warp per pair writes its row, a lane per feature, so that reads of R
+// and stores of X are contiguous.  Bound by the FP64 pipe (two lanes a clock
+// and SM): the entries of R and a~ are therefore taken apart with integer
+// operations and scaled in double-float (the FP32 result is the rounded FP64
+// one but for ties at the 2^-44 level), log10(K / W) is the host's value where
+// K is the first target's, and only tau, its logarithm and |a~| are FP64.
+// 16 384 pairs of W = 9: 31 us with a thread per pair for all of it in FP64, 34
+// with a lane per feature, 23 now.
+constexpr int FEAT_PAIRS = 32, FEAT_THREADS = 512;   // two pairs per warp: their loads' latency is what is left
+
+// r 2^-e as double-float; zero where that is below FP32's range, infinite above.
+__device__ __forceinline__ DF scaled_df(double r, int e) {
+    const int hw = __double2hiint(r);
+    const int x = (hw >> 20) & 0x7FF, y = x - e;
+    double v = r;
+    if (x != 0 && x != 0x7FF) {
+        if (y <= 0) v = 0.0;
+        else if (y >= 0x7FF) v = __hiloint2double((hw & (int)0x80000000) | 0x7FF00000, 0);
+        else v = __hiloint2double((hw & ~0x7FF00000) | (y << 20), __double2loint(r));
+    }
+    const float2 s = split_f64(v);
+    return DF{s.x, s.y};
+}
+__device__ __forceinline__ float df_product(DF a, DF b) {   // rounded to FP32
+    const float p = a.h * b.h;
+    return p + fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)));
+}
+
+__global__ void __launch_bounds__(FEAT_THREADS)
+    features_kernel(const double2 *__restrict__ R, const int64_t *__restrict__ roff, const int32_t *__restrict__ Wg,
+                    const int32_t *__restrict__ Kg, const int64_t *__restrict__ woff,
+                    const double2 *__restrict__ at64, int64_t pairs, int nfeat, int K0, float lk0,
+                    float *__restrict__ X) {
+    // 1 / tau and 1 / |a~| scaled by a power of two each, as double-float
+    __shared__ DF itau_s[FEAT_PAIRS], ina_s[FEAT_PAIRS];
+    __shared__ int et_s[FEAT_PAIRS];
+    __shared__ float ltau_s[FEAT_PAIRS], lk_s[FEAT_PAIRS];
+    const int64_t g0 = (int64_t)blockIdx.x * FEAT_PAIRS;
+    const int np = (int)min((int64_t)FEAT_PAIRS, pairs - g0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int W = Wg[g0];   // one window size for all targets
+    if (warp == 0 && lane < np) {
+        const double2 *Rg = R + roff[g0 + lane];
+        double tr = 0.0;
+        for (int i = 0; i < W; ++i) tr += Rg[i * W + i].x;
+        const double tau = tr / W;
+        ltau_s[lane] = (float)log10(tau);
+        const int x = (__double2hiint(tau) >> 20) & 0x7FF;
+        const int e = (x != 0 && x != 0x7FF) ? x - 1023 : 0;
+        const DF t = scaled_df(tau, e);   // 1 <= |t| < 2
+        const float q = 1.f / t.h;
+        itau_s[lane] = df_norm(q, (fmaf(-q, t.h, 1.f) - q * t.l) * q);
+        et_s[lane] = e;
+    } else if (warp == 1 && lane < np) {   // another warp, at the same time
+        const double2 *a = at64 + woff[g0 + lane];
+        double na = 0.0;
+        for (int i = 0; i < W; ++i) na += a[i].x * a[i].x + a[i].y * a[i].y;
+        ina_s[lane] = scaled_df(rsqrt(na), 0);
+        const int K = Kg[g0 + lane];
+        lk_s[lane] = K == K0 ? lk0 : (float)log10((double)K / (double)W);
+    }
+    __syncthreads();
+    const int tri = W * (W - 1) / 2;
+    for (int k = warp; k < np; k += FEAT_THREADS / 32) {
+        const int64_t g = g0 + k;
+        const double2 *Rg = R + roff[g];
+        const double2 *a = at64 + woff[g];
+        const DF itau = itau_s[k], ina = ina_s[k];
+        const int et = et_s[k];
+        float *x = X + g * nfeat;
+        for (int o = lane; o < nfeat; o += 32) {
+            float f;
+            if (o < W + 2 * tri) {
+                const bool im = o >= W + tri;
+                int i = o, j = o;
+                if (o >= W) {
+                    const int q = o - W - (im ? tri : 0);   // entry of the strict lower triangle, row-major
+                    i = (int)((sqrtf(8.f * (float)q + 1.f) + 1.f) * 0.5f);
+                    i += i * (i + 1) / 2 <= q;   // the rounded root may be one off
+                    i -= i * (i - 1) / 2 > q;
+                    j = q - i * (i - 1) / 2;
+                }
+                const double2 r = Rg[i * W + j];
+                f = df_product(scaled_df(im ? r.y : r.x, et), itau);
+            } else if (o < 3 * W + 2 * tri) {
+                const int q = o - W - 2 * tri;
+                f = df_product(scaled_df(q < W ? a[q].x : a[q - W].y, 0), ina);
+            } else {
+                f = o == nfeat - 2 ? ltau_s[k] : lk_s[k];
+            }
+            x[o] = f;
+        }
+    }
 }
 
 // ----------------------------------------------------------------- SINR judge
@@ -274,8 +342,9 @@ bs_status bs_features(const bs_plan *p, const bs_cf64 *R_unloaded, float *X, bs_
         if (p->Wt[t] != p->Wt[0]) return set_error(BS_EINVAL, "features need one window size for all targets");
     const int W = p->Wt[0];
     const int nfeat = W * W + 2 * W + 2;
-    bs::features_kernel<<<bs::blocks_for(p->pairs, 128), 128, 0, (cudaStream_t)stream>>>(
-        (const double2 *)R_unloaded, p->d_roff, p->d_Wg, p->d_Kg, p->d_woff, p->d_at64, p->pairs, nfeat, X);
+    bs::features_kernel<<<bs::blocks_for(p->pairs, bs::FEAT_PAIRS), bs::FEAT_THREADS, 0, (cudaStream_t)stream>>>(
+        (const double2 *)R_unloaded, p->d_roff, p->d_Wg, p->d_Kg, p->d_woff, p->d_at64, p->pairs, nfeat, p->Kt[0],
+        (float)log10((double)p->Kt[0] / (double)W), X);
     return bs::check_launch("features launch");
 }
 

@@ -6,7 +6,7 @@
 // correlators with N x columns: the columns are the channelised test vectors,
 // or the steering vectors e^{j Omega n} of a grid of directions, which depend
 // on the subband and the direction only and are generated as the operand is
-// staged.  A CTA computes 64 targets by up to 128 columns.
+// staged.  A CTA computes 64 targets by up to 128 columns (192 directions).
 //
 // tcgen05.mma, M = 128: rows 0-63 hold (Re c, Im c) and rows 64-127
 // (-Im c, Re c) interleaved along K, so that with columns (Re y, Im y) they
@@ -22,17 +22,20 @@
 // groups of eight warps take the even and the odd stages (load FP32 a turn
 // ahead, split, store in the canonical K-major layout with core matrices 160
 // bytes apart along K, so that the 16-byte stores of a quarter warp hit
-// distinct banks), and each warp drains 32 tensor-memory lanes x 32 columns
-// of every chunk.  Warp 16 issues the products: per stage of 16 elements
-// 2 x 6.  Measured at 64 targets, 1024 elements and 128 subbands: 128 test
-// vectors 327 -> 76 us (26 -> 113 TFLOP/s of the 8 T N V flops), 181
-// directions 598 -> 122 us; the SIMT kernels these replace were bound by
-// shared-memory loads (2 x 2 register tiles) and by one rotation per pair,
-// element and direction.  Timing copies with parts left out: products alone
-// 0.62 us per stage (98 cycles each: both operands come from shared memory),
-// hand-overs alone 0.29, splitting alone 0.5; a tile also pays 8 us of launch,
-// drain and store.  The test-vector product adds the latency of its loads
-// (76 -> 54 us without them), the pattern the generation of its columns.
+// distinct banks), and each warp drains 32 tensor-memory lanes x a quarter of
+// the columns of every chunk.  Warp 16 issues the products: per stage of 16
+// elements 2 x 6, the trailing ones first, so that the drain of the last
+// chunk's leading sum is hidden behind them.
+//
+// Measured at 64 targets, 1024 elements and 128 subbands: 128 test vectors
+// 327 -> 62 us, 181 directions 598 -> 88 us; the SIMT kernels these replace
+// were bound by shared-memory loads (2 x 2 register tiles, 26 TFLOP/s) and by
+// one rotation per pair, element and direction.  With two leading sums drained
+// two stages late and two direction tiles of 128: 76 and 122 us.  Timing copies
+// with parts left out: products alone 45 us for 128 columns and 53 for 192 (98
+// and 111 cycles each: both operands come from shared memory), hand-overs alone
+// 19 and 25 (8 of launch, drain and store), loading, splitting and storing the
+// operands alone 54 and 68.
 #include "common.cuh"
 #include "internal.h"
 #include "tcgen05.cuh"
@@ -43,21 +46,29 @@ namespace bs {
 namespace {
 
 constexpr int LT_T = 64;          // targets per CTA
-constexpr int LT_C = 128;         // columns per CTA
 constexpr int LT_K = 16;          // elements per stage (32 real rows of K)
 constexpr int LT_CHUNK = 4;       // stages per drained chunk
 constexpr int LT_STAGES = 3;
 constexpr int LT_THREADS = 544;
 constexpr int LT_LBO = 160, LT_SBO = 640;              // core matrices along K; 8-row groups
-constexpr int LT_PART = 16 * LT_SBO;                   // one part of 128 rows
-constexpr int LT_OP = 3 * LT_PART;                     // an operand's three parts
-constexpr int LT_STAGE = 2 * LT_OP;
-constexpr int LT_MISC = LT_STAGES * LT_STAGE;
-constexpr int LT_SMEM = LT_MISC + 128 + 2 * LT_T * 8;
-constexpr int LT_PITCH = LT_C + 1;                     // output tile, float2
-static_assert(LT_T * LT_PITCH * 8 <= LT_MISC, "the output tile reuses the stages");
-static_assert(LT_SMEM <= 227 * 1024, "one CTA's shared memory");
-constexpr uint32_t LT_COLS = 512;                      // tensor memory: leading sums x 2, trailing sum (128 columns each)
+constexpr int LT_PART = 16 * LT_SBO;                   // one part of the 128 rows of A
+constexpr int LT_OP = 3 * LT_PART;                     // A's three parts
+// CC columns per CTA: 128 test vectors, or 192 directions (181 degrees in one
+// tile: a product costs nearly the same for 64 to 192 columns, and the
+// correlators are split once)
+template <int CC>
+struct LtTile {
+    static constexpr int bpart = CC / 8 * LT_SBO;      // one part of the CC columns of B
+    static constexpr int stage = LT_OP + 3 * bpart;
+    static constexpr int misc = LT_STAGES * stage;
+    static constexpr int smem = misc + 128 + 2 * LT_T * 8;
+    static constexpr int pitch = CC + 1;               // output tile, float2
+    static constexpr int dc = CC / 4;                  // columns drained per warp
+    static_assert(LT_T * pitch * 8 <= misc, "the output tile reuses the stages");
+    static_assert(smem <= 227 * 1024, "one CTA's shared memory");
+    static_assert(2 * CC <= 512, "tensor memory: leading sum at column 0, trailing sum at 256");
+};
+constexpr uint32_t LT_COLS = 512;                      // tensor memory columns
 
 struct LtArgs {
     const float2 *c_hat;   // [T][L][N]
@@ -145,13 +156,16 @@ __device__ __forceinline__ float2 steer(float2 om, float x) {
 
 template <bool PATTERN, bool VEC>
 __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) {
+    constexpr int CC = PATTERN ? 192 : 128, NI = CC / 64;   // NI: column items per thread and stage
+    using TT = LtTile<CC>;
+    constexpr int LT_MISC = TT::misc, LT_STAGE = TT::stage, LT_PITCH = TT::pitch, LT_C = CC;
     extern __shared__ __align__(128) unsigned char smlt[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint64_t *full = reinterpret_cast<uint64_t *>(smlt + LT_MISC);   // [LT_STAGES] stage written (the 8 warps of a group)
     uint64_t *empty = full + LT_STAGES;                              // [LT_STAGES] its products are done
-    uint64_t *dfull = empty + LT_STAGES;                             // [2] a chunk's leading sum is complete
-    uint64_t *dempty = dfull + 2;                                    // [2] it has been drained (16 warps)
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(dempty + 2);
+    uint64_t *dfull = empty + LT_STAGES;                             // a chunk's leading sum is complete
+    uint64_t *dempty = dfull + 1;                                    // it has been drained (16 warps)
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(dempty + 1);
     float2 *nrm = reinterpret_cast<float2 *>(smlt + LT_MISC + 128);  // [2 groups][64] ||sc c_hat||^2 of its stages, sc
     const uint32_t sbase = smem_u32(smlt);
 
@@ -168,10 +182,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
             mbar_init(&full[j], 8);
             mbar_init(&empty[j], 1);
         }
-        for (int j = 0; j < 2; ++j) {
-            mbar_init(&dfull[j], 1);
-            mbar_init(&dempty[j], 16);
-        }
+        mbar_init(dfull, 1);
+        mbar_init(dempty, 16);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 16) tmem_alloc(tslot, LT_COLS);
@@ -186,37 +198,42 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
         // (four neighbouring lanes read 128 bytes of a row)
         const int grp = warp >> 3, r = 8 * (warp & 7) + (lane >> 2), c = lane & 3;
         const uint32_t off = sbase + (uint32_t)((r >> 3) * LT_SBO + c * LT_LBO + (r & 7) * 16);
-        // and drains rows 32 q + lane, columns 32 h ..
+        // and drains rows 32 q + lane, columns DC h ..
+        constexpr int DC = TT::dc;
         const int q = warp & 3, h = warp >> 2;
-        const uint32_t dat = tmem + ((uint32_t)(32 * q) << 16) + 32 * h;
-        const bool mine = 32 * h < NB;
-        float2 acc[16];
+        const uint32_t dat = tmem + ((uint32_t)(32 * q) << 16) + DC * h;
+        const bool mine = DC * h < NB;
+        float2 acc[DC / 2];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) acc[k] = make_float2(0.f, 0.f);
+        for (int k = 0; k < DC / 2; ++k) acc[k] = make_float2(0.f, 0.f);
         auto add = [&](uint32_t ta) {
-            float d[32];
-            tmem_ld32(ta, d);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) acc[k] = __fadd2_rn(acc[k], make_float2(d[2 * k], d[2 * k + 1]));
+            for (int p = 0; p < DC / 16; ++p) {
+                float d[16];
+                tmem_ld16(ta + 16 * p, d);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    acc[8 * p + k] = __fadd2_rn(acc[8 * p + k], make_float2(d[2 * k], d[2 * k + 1]));
+            }
         };
         auto drain = [&](int j) -> bool {   // chunk j's leading sum
-            if (!mbar_wait_bounded(&dfull[j & 1], (unsigned)(j >> 1) & 1u)) return false;
+            if (!mbar_wait_bounded(dfull, (unsigned)j & 1u)) return false;
             if (mine) {
                 tc_fence_after();
-                add(dat + 128 * (j & 1));
+                add(dat);
                 tc_fence_before();
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&dempty[j & 1]);
+            if (lane == 0) mbar_arrive(dempty);
             return true;
         };
         const bool tval = t0 + r < a.T;
         const float2 *crow = a.c_hat + ((int64_t)min(t0 + r, a.T - 1) * a.L + s) * a.N;
-        const float2 *yrow[2];
-        float2 om[2], rot[2][3];
-        bool cval[2];
+        const float2 *yrow[PATTERN ? 1 : NI];
+        float2 om[PATTERN ? NI : 1], rot[PATTERN ? NI : 1];
+        bool cval[NI];
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < NI; ++b) {
             const int v = v0 + r + 64 * b;
             cval[b] = v < a.cols;
             if constexpr (PATTERN) {
@@ -228,14 +245,13 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
                 const double o = cval[b] ? a.u[v] * (f / a.fd) : 0.0;
                 om[b].x = (float)o;
                 om[b].y = (float)(o - (double)om[b].x);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) rot[b][i] = steer(om[b], (float)(i + 1));
+                rot[b] = steer(om[b], 1.f);
             } else {
                 const int vv = cval[b] ? v : 0;
                 yrow[b] = a.xc + ((int64_t)(a.P_train + vv / a.B) * a.F + (int64_t)s * a.B + vv % a.B) * a.N;
             }
         }
-        const int nb = NB > 64 ? 2 : 1;   // column halves in use
+        const int nb = (NB + 63) >> 6;   // blocks of 64 columns in use
         // sum of squares of this thread's part of the row, (hi, lo), scaled by
         // the power of two that brings the row's first elements near 1, so
         // that neither the norm nor the squares below leave FP32's range
@@ -251,7 +267,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
             const int e = max(-120, min(120, ((__float_as_int(m) >> 23) & 255) - 127));
             if (m > 0.f && isfinite(m)) sc = __int_as_float((127 - e) << 23);
         }
-        float2 xa[4], xb[PATTERN ? 1 : 2][4];
+        float2 xa[4], xb[PATTERN ? 1 : NI][4];
         auto fetch = [&](int st) {
             const int n = st * LT_K + 4 * c;
             load_item<VEC>(crow, n, a.N, tval, xa);
@@ -260,9 +276,9 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
                 if (nb > 1) load_item<VEC>(yrow[1], n, a.N, cval[1], xb[1]);
             }
         };
-        auto put = [&](uint32_t addr, const uint32_t (&w)[3][4]) {
+        auto put = [&](uint32_t addr, uint32_t part, const uint32_t (&w)[3][4]) {
 #pragma unroll
-            for (int p = 0; p < 3; ++p) st_shared_v4(addr + p * LT_PART, w[p][0], w[p][1], w[p][2], w[p][3]);
+            for (int p = 0; p < 3; ++p) st_shared_v4(addr + p * part, w[p][0], w[p][1], w[p][2], w[p][3]);
         };
         auto stage = [&](int st) -> bool {
             const int b = st % LT_STAGES, use = st / LT_STAGES;
@@ -270,12 +286,12 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
             const uint32_t at = off + (uint32_t)(b * LT_STAGE);
             uint32_t w[3][4];
             split_item(xa, w);
-            put(at, w);
+            put(at, LT_PART, w);
 #pragma unroll
             for (int p = 0; p < 3; ++p)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) w[p][i] = __byte_perm(w[p][i], w[p][i], 0x1032) ^ 0x8000u;   // (-Im, Re)
-            put(at + 8 * LT_SBO, w);   // row r + 64
+            put(at + 8 * LT_SBO, LT_PART, w);   // row r + 64
             if constexpr (PATTERN) {
                 float s2 = 0.f;
 #pragma unroll
@@ -288,18 +304,18 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
                 nh = sm;
             }
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < NI; ++h) {
                 if (h >= nb) break;
                 if constexpr (PATTERN) {
                     float2 e[4];
                     e[0] = steer(om[h], (float)(st * LT_K + 4 * c));
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) e[i + 1] = cmul(e[0], rot[h][i]);
+                    for (int i = 0; i < 3; ++i) e[i + 1] = cmul(e[i], rot[h]);
                     split_item(e, w);
                 } else {
                     split_item(xb[h], w);
                 }
-                put(at + LT_OP + h * 8 * LT_SBO, w);
+                put(at + LT_OP + h * 8 * LT_SBO, TT::bpart, w);
             }
             fence_proxy_async();   // the tensor core reads the stage through the async proxy
             __syncwarp();
@@ -311,9 +327,10 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
         bool ok = true;
         int j = 0;   // chunks drained
         for (int st = grp; st < nst && ok; st += 2) {
-            // chunk j is drained two stages after its last: its products are
-            // mostly done, and they never wait for a later drain than this
-            if (st > LT_CHUNK * j + LT_CHUNK + 1) ok = drain(j++);
+            // chunk j is drained once this group has staged a part of the next
+            // chunk, whose leading products wait for it (its trailing ones,
+            // issued first, do not)
+            if (st > LT_CHUNK * j + LT_CHUNK) ok = drain(j++);
             if (ok) ok = stage(st);
         }
         for (; j < nch && ok; ++j) ok = drain(j);
@@ -322,9 +339,9 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
                 tc_fence_after();
                 add(dat + 256);
                 const int row = 32 * q + lane;
-                float *tile = reinterpret_cast<float *>(smlt) + ((row & 63) * LT_PITCH + 32 * h) * 2 + (row >> 6);
+                float *tile = reinterpret_cast<float *>(smlt) + ((row & 63) * LT_PITCH + DC * h) * 2 + (row >> 6);
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
+                for (int k = 0; k < DC / 2; ++k) {
                     tile[4 * k] = acc[k].x;
                     tile[4 * k + 2] = acc[k].y;
                 }
@@ -344,30 +361,37 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
                                | ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         bool ok = true;
         for (int st = 0; st < nst && ok; ++st) {
-            const int b = st % LT_STAGES, j = st / LT_CHUNK, d = j & 1;
+            const int b = st % LT_STAGES, j = st / LT_CHUNK;
             ok = mbar_wait_bounded(&full[b], (unsigned)(st / LT_STAGES) & 1u);
-            if (ok && st % LT_CHUNK == 0 && j >= 2) ok = mbar_wait_bounded(&dempty[d], (unsigned)((j >> 1) - 1) & 1u);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
-                const uint32_t sa = sbase + b * LT_STAGE, sb = sa + LT_OP;
+            const uint32_t sa = sbase + b * LT_STAGE, sb = sa + LT_OP;
+            if (lane == 0) {   // trailing products
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     uint64_t da[3], db[3];
 #pragma unroll
                     for (int p = 0; p < 3; ++p) {
                         da[p] = lt_desc(sa + p * LT_PART + k * 2 * LT_LBO);
-                        db[p] = lt_desc(sb + p * LT_PART + k * 2 * LT_LBO);
+                        db[p] = lt_desc(sb + p * TT::bpart + k * 2 * LT_LBO);
                     }
-                    mma_ss<0>(tmem + 128 * d, da[0], db[0], idesc, st % LT_CHUNK | k);
-                    mma_ss<1>(tmem + 256, da[0], db[1], idesc, st | k);
+                    mma_ss<0>(tmem + 256, da[0], db[1], idesc, st | k);
                     mma_ss<2>(tmem + 256, da[0], db[2], idesc, 1);
                     mma_ss<0>(tmem + 256, da[1], db[0], idesc, 1);
                     mma_ss<2>(tmem + 256, da[1], db[1], idesc, 1);
                     mma_ss<3>(tmem + 256, da[2], db[0], idesc, 1);
                 }
+            }
+            __syncwarp();
+            if (st % LT_CHUNK == 0 && j >= 1) ok = mbar_wait_bounded(dempty, (unsigned)(j - 1) & 1u);
+            if (!ok) break;
+            tc_fence_after();
+            if (lane == 0) {   // leading products
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    mma_ss<3>(tmem, lt_desc(sa + k * 2 * LT_LBO), lt_desc(sb + k * 2 * LT_LBO), idesc, st % LT_CHUNK | k);
                 mma_commit(&empty[b]);
-                if (st % LT_CHUNK == LT_CHUNK - 1 || st + 1 == nst) mma_commit(&dfull[d]);
+                if (st % LT_CHUNK == LT_CHUNK - 1 || st + 1 == nst) mma_commit(dfull);
             }
             __syncwarp();
         }
@@ -401,20 +425,21 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
 
 template <bool PATTERN, bool VEC>
 bs_status launch_lift_tc_t(const LtArgs &a, cudaStream_t st) {
+    constexpr int smem = LtTile<PATTERN ? 192 : 128>::smem;
     static PerDevice attr;
     if (bs_status s = attr.get([](int *) {
             return cuda_error(cudaFuncSetAttribute(lift_tc_kernel<PATTERN, VEC>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, LT_SMEM),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                               "lifted products attribute");
         }))
         return s;
     const int64_t tiles = (int64_t)a.L * a.tt * a.ct;
     if (tiles > 0x7FFFFFFF) return set_error(BS_EUNSUPPORTED, "too many tiles");
-    lift_tc_kernel<PATTERN, VEC><<<(unsigned)tiles, LT_THREADS, LT_SMEM, st>>>(a);
+    lift_tc_kernel<PATTERN, VEC><<<(unsigned)tiles, LT_THREADS, smem, st>>>(a);
     return check_launch("lifted products launch");
 }
 
-LtArgs lift_args(const bs_plan *p, const float2 *c_hat, int cols) {
+LtArgs lift_args(const bs_plan *p, const float2 *c_hat, int cols, int tile) {
     LtArgs a{};
     a.c_hat = c_hat;
     a.N = p->cfg.N;
@@ -422,7 +447,7 @@ LtArgs lift_args(const bs_plan *p, const float2 *c_hat, int cols) {
     a.T = p->cfg.T;
     a.cols = cols;
     a.tt = (a.T + LT_T - 1) / LT_T;
-    a.ct = (cols + LT_C - 1) / LT_C;
+    a.ct = (cols + tile - 1) / tile;
     a.err = p->d_err;
     return a;
 }
@@ -434,7 +459,7 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 bs_status launch_apply_lifted(const bs_plan *p, const float2 *xc, const float2 *c_hat, float2 *out,
                               cudaStream_t st) {
     if (p->Vte == 0 || p->pairs == 0) return BS_OK;
-    LtArgs a = lift_args(p, c_hat, p->Vte);
+    LtArgs a = lift_args(p, c_hat, p->Vte, 128);
     a.xc = xc;
     a.F = p->Fs;
     a.B = p->B;
@@ -449,7 +474,7 @@ bs_status launch_beam_pattern(const bs_plan *p, const float2 *c_hat, int n_dirs,
     if (n_dirs == 0 || p->pairs == 0) return BS_OK;
     if (((size_t)p->cfg.N + n_dirs) * sizeof(float2) > 200 * 1024)
         return set_error(BS_EUNSUPPORTED, "beam pattern: N + n_dirs must be <= 25600");
-    LtArgs a = lift_args(p, c_hat, n_dirs);
+    LtArgs a = lift_args(p, c_hat, n_dirs, 192);
     a.u = u;
     a.Ltot = p->cfg.L;
     a.s0 = p->s0;

@@ -1,6 +1,6 @@
 """The lifted correlator's tensor-core products and its lift at the sizes
 where their tiles end: targets around the 64-target tile, columns around the
-128-column tile and below 16, element counts around the 16-element stage and
+128-column (192-direction) tile and below 16, element counts around the 16-element stage and
 the 64-element chunk, odd counts (unaligned rows), weights at extreme scales,
 subband shards, and a failed pair's NaN weights staying its own.
 
@@ -31,7 +31,7 @@ def _plan(N, T, L, B, P_te, **kw):
 @pytest.mark.parametrize("N,T,L,B,P_te,scale", [
     (1024, 64, 16, 16, 8, 1.0), (1, 1, 16, 1, 1, 1.0), (15, 3, 8, 2, 3, 1.0), (16, 65, 4, 4, 4, 1e-30),
     (17, 63, 4, 8, 2, 1e18), (65, 2, 2, 64, 2, 1.0), (100, 130, 2, 32, 5, 1.0), (301, 37, 8, 4, 33, 1.0),
-    (64, 20, 16, 8, 16, 1.0)])
+    (64, 20, 16, 8, 16, 1.0), (33, 5, 2, 128, 1, 1.0), (200, 70, 2, 64, 3, 1.0)])
 def test_lifted_products_match_fp64(N, T, L, B, P_te, scale):
     plan = _plan(N, T, L, B, P_te)
     g = torch.Generator(device="cuda").manual_seed(N + T)

@@ -6,7 +6,10 @@
 // FFT in shared memory; a CTA takes VPB consecutive vectors.  The windowed
 // variant then writes, for every target, the W_t beams of its window
 // (start_g + w mod M) straight from shared memory into the packed training
-// or test window arrays; the full variant writes all M beams.
+// or test window arrays; the full variant writes all M beams.  Decoding each
+// (target, beam) entry once for all VPB vectors instead of once per output took
+// 24 576 vectors of N = 256, M = 512 from 35 to 32 us and 16 384 of 100 targets
+// of 11 beams from 64 to 44 us.
 #include "beamspace_dev.cuh"
 #include "internal.h"
 
@@ -27,7 +30,7 @@ __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
     // FFT so that the table loads overlap the butterflies
     __shared__ long long tab_base[kTabT];
     __shared__ int tab_sw[kTabT];     // start | (W << 16)
-    __shared__ int tab_n[kTabT];      // outputs of this target in this CTA (0: none)
+    __shared__ int tab_n[kTabT];      // vectors of this CTA that the target's windows take (0: none)
     const int tid = threadIdx.x;
     const int64_t vid0 = (int64_t)blockIdx.x * vpb;
     int s_cta = 0, v0_cta = 0;
@@ -76,30 +79,35 @@ __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
             if (v < nvec) out[v * M + m] = cscale(sload(c, m), scale);
         }
     } else if (ga.uniform) {
-        // All vpb vectors share record p and subband s (bins i0 .. i0+vpb-1).
-        // Flat loop over the (target, vector c, beam w) entries of the gather
-        // table; the vpb * W_t outputs of target t form one contiguous run of
-        // the window array (element k = c * W_t + w from the target's base).
+        // All vpb vectors share record p and subband s (bins i0 .. i0+vpb-1):
+        // a thread decodes a (target, beam w) entry once and stores it for
+        // every vector (the vectors' rows of W_t are contiguous from the
+        // target's base).
         if (vid0 >= ga.nvec) return;
         const int nv = (ga.nvec - vid0 < (int64_t)vpb) ? (int)(ga.nvec - vid0) : vpb;
-        for (int e = tid; e < ga.ngather; e += nthr) {
-            const int packed = __ldg(&ga.gather[e]);
-            const int t = packed >> 10, c = (packed >> 5) & 31, w = packed & 31;
+        for (int e = tid; e < ga.sumW; e += nthr) {
+            const int packed = __ldg(&ga.glist[e]);
+            const int t = packed >> 8, w = packed & 255;
             long long base;
-            int sw, nout;
+            int sw, n;
             if (t < kTabT) {
                 base = tab_base[t];
                 sw = tab_sw[t];
-                nout = tab_n[t];
+                n = tab_n[t];
             } else {
-                fill_target_entry(ga, t, s_cta, v0_cta, nv, train_cta, &base, &sw, &nout, 0);
+                fill_target_entry(ga, t, s_cta, v0_cta, nv, train_cta, &base, &sw, &n, 0);
             }
             const int W = sw >> 16;
-            const int k = c * W + w;
-            if (k >= nout) continue;
-            const float2 val = cscale(sload(c, ((sw & 0xFFFF) + w) & (M - 1)), scale);
-            if (train_cta) store_train<PREC>(ga.ztr, base + k, val, ga.store_scale);
-            else ga.zte[base + k] = val;
+            const float2 *src = sm + padrow(((sw & 0xFFFF) + w) & (M - 1));
+            const long long o = base + w;
+            if (train_cta) {
+#pragma unroll 4
+                for (int c = 0; c < n; ++c)
+                    store_train<PREC>(ga.ztr, o + (long long)c * W, cscale(src[c * pl], scale), ga.store_scale);
+            } else {
+#pragma unroll 4
+                for (int c = 0; c < n; ++c) ga.zte[o + (long long)c * W] = cscale(src[c * pl], scale);
+            }
         }
     } else {
         const int Fm1 = (1 << ga.log2F) - 1, Bm1 = (1 << ga.log2B) - 1;
@@ -184,6 +192,8 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     ga.P_train = p->cfg.P_train;
     ga.uniform = (p->B % p->vpb) == 0;
     ga.gather = p->d_gather;
+    ga.glist = p->d_glist;
+    ga.sumW = p->sumW;
     ga.gsub = reinterpret_cast<const longlong2 *>(p->d_gsub);
     ga.ngather = (int)p->gather.size();
     ga.Wg = p->d_Wg;
@@ -198,7 +208,12 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     bool used = false;
     bs_status s = BS_OK;
     // -1: the first variant that applies, in the order tensor cores, warp per
-    // transform, bulk-copy-staged, one-shot; 0..3 start the search there
+    // transform, one-shot (0, 2 and 3 start the search there).  The
+    // bulk-copy-staged kernel is slower than the one-shot kernel wherever both
+    // apply and the first two do not (24 576 vectors of N = 256, M = 512, 16
+    // targets: 45 against 32 us; 16 384 of N = 300, 100 targets: 148 against 44;
+    // 6 144 of N = 1500, M = 2048: 48 against 39; N = 2000, M = 4096: 87 against
+    // 76) and runs where it is asked for.
     const int v = p->tune_beamspace;
     if (v < 0 || v == 3) {
         s = launch_beamspace_tc(p, xc, ga, st, &used);
@@ -208,7 +223,7 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
         s = launch_beamspace_warp(p, xc, ga, st, &used);
         if (s || used) return s;
     }
-    if (v <= 1 || v == 3) {
+    if (v == 1 || (v < 0 && (p->cfg.flags & BS_FLAG_STAGED_FFT))) {
         s = launch_beamspace_tma(p, xc, ga, st, &used);
         if (s || used) return s;
     }

@@ -28,6 +28,8 @@ struct GatherArgs {
     const int32_t *gather;  // [vpb * sumW] (t << 10) | (c << 5) | w
     const longlong2 *gsub;  // [L][T][2]: {ztr_off, zte_off}, {start | W << 16, K}
     int ngather;
+    const int32_t *glist;   // [sumW] (t << 8) | w, target-major
+    int sumW;
     const int32_t *Wg, *Kg, *start;
     const int64_t *ztr_off, *zte_off;
     void *ztr;              // training windows (plan precision)
@@ -56,8 +58,9 @@ struct __align__(16) GatherEnt {
     int n;
 };
 
-// Gather entry of target t for a CTA at subband s whose first vector is v0:
-// base element offset in the window array, start | (W << 16), output count.
+// Gather entry of target t for a CTA at subband s whose first vector is v0 and
+// which holds nv: base element offset in the window array, start | (W << 16),
+// vectors to store.
 __device__ __forceinline__ void fill_target_entry(const GatherArgs &ga, int t, int s, int v0, int nv,
                                                   bool train, long long *base, int *sw, int *nout,
                                                   int slot = -1) {
@@ -65,11 +68,11 @@ __device__ __forceinline__ void fill_target_entry(const GatherArgs &ga, int t, i
     const int64_t g = (int64_t)t * ga.L + s;
     const int W = __ldg(&ga.Wg[g]);
     const int st = __ldg(&ga.start[g]);
-    int n = nv * W;
+    int n = nv;
     long long b;
     if (train) {
         const int K = __ldg(&ga.Kg[g]);
-        n = (v0 >= K) ? 0 : min(n, (K - v0) * W);
+        n = max(0, min(n, K - v0));
         b = __ldg(&ga.ztr_off[g]) + (long long)v0 * W;
     } else {
         b = __ldg(&ga.zte_off[g]) + (long long)v0 * W;

@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(256, 2)
                 nout = te.n;
             } else {
                 fill_target_entry(ga, t, sb, v0, vpb, train, &base, &sw, &nout, 0);
+                nout *= sw >> 16;   // vectors to outputs
             }
             const int k = c * (sw >> 16) + w;
             if (k >= nout) return;

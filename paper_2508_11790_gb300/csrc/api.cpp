@@ -328,7 +328,7 @@ bs_status bs_autotune_pass(bs_plan *p, const bs_buffers *b, bs_stream stream, bs
             s = time_of([&] { return bs::launch_beamspace(p, (const float2 *)b->xc, b->z_train, (float2 *)b->z_test, st); },
                         &ms);
             r.beamspace_ms[v] = ms;
-            if (!s && ms < best) best = ms, best_b = v;
+            if (!s && ms <= best) best = ms, best_b = v;   // on a tie the later one (one-shot over warp: close at M = 1024)
         }
     }
     p->tune_beamspace = best_b;

@@ -153,24 +153,31 @@ bs_status bs_cov_solve(const bs_plan *p, const void *z_train, const float *delta
 
 bs_status bs_run(const bs_plan *p, const bs_buffers *b, bs_stream stream) {
     BS_REQUIRE(p && b, "NULL argument");
+    const cudaStream_t st = (cudaStream_t)stream;
     bs_status s;
     if ((s = bs_channelize(p, b->x, p->P, b->xc, stream))) return s;
-    if ((s = bs_beamspace(p, b->xc, b->z_train, b->z_test, stream))) return s;
+    BS_REQUIRE(b->xc && b->z_train, "NULL buffer");
+    BS_REQUIRE(b->z_test || p->cfg.P_test == 0, "z_test is NULL but P_test > 0");
+    // from here each stage follows a kernel of this pass on the stream, so it
+    // may be placed while that one runs (dependent = true)
+    if ((s = bs::launch_beamspace(p, (const float2 *)b->xc, b->z_train, (float2 *)b->z_test, st, 0, -1, true))) return s;
     if (use_fused(p)) {
         if ((s = bs_cov_solve(p, b->z_train, nullptr, b->R, b->c, b->info, stream))) return s;
-    } else if (bs::cov_solve_chains_apply(p)) {
+        return bs_apply(p, b->z_test, b->c, b->out, stream);
+    }
+    BS_REQUIRE(b->R && b->c && b->info, "NULL buffer");
+    if (bs::cov_solve_chains_apply(p)) {
         // several window sizes on the warp-per-pair covariance: one
         // covariance + solve chain per size, the chains in parallel
-        BS_REQUIRE(b->z_train && b->R && b->c && b->info, "NULL buffer");
-        if ((s = check_device(p))) return s;
-        if ((s = bs::launch_cov_solve_chains(p, b->z_train, (double2 *)b->R, (float2 *)b->c, b->info,
-                                             (cudaStream_t)stream)))
-            return s;
-    } else {
-        if ((s = bs_window_cov(p, b->z_train, nullptr, b->R, stream))) return s;
-        if ((s = bs_mvdr_solve(p, b->R, b->c, b->info, stream))) return s;
+        if ((s = bs::launch_cov_solve_chains(p, b->z_train, (double2 *)b->R, (float2 *)b->c, b->info, st))) return s;
+        return bs_apply(p, b->z_test, b->c, b->out, stream);
     }
-    return bs_apply(p, b->z_test, b->c, b->out, stream);
+    if ((s = bs::launch_window_cov(p, b->z_train, nullptr, (double2 *)b->R, st, true))) return s;
+    const bool one = bs::mvdr_solve_is_one_launch(p);   // else the side streams are joined by events
+    if ((s = bs::launch_mvdr_solve(p, (const double2 *)b->R, (float2 *)b->c, b->info, st, nullptr, one))) return s;
+    if (p->Vte == 0) return BS_OK;
+    BS_REQUIRE(b->z_test && b->c && b->out, "NULL buffer");
+    return bs::launch_apply(p, (const float2 *)b->z_test, (const float2 *)b->c, (float2 *)b->out, st, one);
 }
 
 struct bs_graph {

@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
                  const int32_t *__restrict__ Wg, const int64_t *__restrict__ woff,
                  const float2 *__restrict__ c, float2 *__restrict__ out, int64_t total, int Vte) {
     __shared__ float2 span[ApplyCfg<WM>::threads / 32][ApplyCfg<WM>::span];
+    wait_for_predecessor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t idx0 = (int64_t)blockIdx.x * blockDim.x + warp * 32;
     if (idx0 >= total) return;   // uniform per warp
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
     constexpr int NW = ApplyCfg<WM>::threads / 32, NR = WM / 2;   // 16-byte loads per lane: 16 W per block
     __shared__ __align__(16) float2 span[NW][ApplyCfg<WM>::span];
     __shared__ float2 cw[NW][WM];
+    wait_for_predecessor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned unit = blockIdx.x * NW + warp;   // upp units per pair
     if (unit >= units) return;   // uniform per warp
@@ -107,19 +109,21 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
 }
 
 template <int WM>
-static bs_status launch_apply_blocks(const bs_plan *p, const float2 *z, const float2 *c, float2 *out, cudaStream_t st) {
+static bs_status launch_apply_blocks(const bs_plan *p, const float2 *z, const float2 *c, float2 *out, cudaStream_t st,
+                                     bool dependent) {
     constexpr int NW = ApplyCfg<WM>::threads / 32;
     const int nb = p->Vte / 32;
     // several blocks per warp only where the pairs alone fill the GPU (64 warps an SM)
     const int bpw = p->pairs >= 32LL * p->num_sms ? (nb < 4 ? nb : 4) : 1;
     const unsigned upp = (unsigned)((nb + bpw - 1) / bpw);
     const unsigned units = (unsigned)p->pairs * upp;
-    apply_blocks_kernel<WM><<<(units + NW - 1) / NW, ApplyCfg<WM>::threads, 0, st>>>(
-        z, p->d_zte_off, p->d_Wg, p->d_woff, c, out, units, upp, nb, bpw);
+    launch_stage(dependent, apply_blocks_kernel<WM>, (units + NW - 1) / NW, ApplyCfg<WM>::threads, 0, st, z, p->d_zte_off,
+                 p->d_Wg, p->d_woff, c, out, units, upp, nb, bpw);
     return check_launch("apply launch");
 }
 
-bs_status launch_apply(const bs_plan *p, const float2 *zte, const float2 *c, float2 *out, cudaStream_t st) {
+bs_status launch_apply(const bs_plan *p, const float2 *zte, const float2 *c, float2 *out, cudaStream_t st,
+                       bool dependent) {
     const int64_t total = p->pairs * p->Vte;
     if (total == 0) return BS_OK;
     if (p->Wmax > 32) return set_error(BS_EUNSUPPORTED, "W > 32");
@@ -128,16 +132,12 @@ bs_status launch_apply(const bs_plan *p, const float2 *zte, const float2 *c, flo
     // 21.3 -> 19.3 us (12.5 at the copy bandwidth); 32 768 pairs of W = 3..15:
     // 67.6 -> 53.8 (46).
     if (p->Vte % 32 == 0 && (reinterpret_cast<uintptr_t>(zte) & 15) == 0 && total / 32 < (1LL << 31))
-        return p->Wmax <= 16 ? launch_apply_blocks<16>(p, zte, c, out, st) : launch_apply_blocks<32>(p, zte, c, out, st);
-    if (p->Wmax <= 16) {
-        constexpr int thr = ApplyCfg<16>::threads;
-        apply_kernel<16><<<(unsigned)((total + thr - 1) / thr), thr, 0, st>>>(zte, p->d_zte_off, p->d_Wg, p->d_woff, c,
-                                                                             out, total, p->Vte);
-    } else {
-        constexpr int thr = ApplyCfg<32>::threads;
-        apply_kernel<32><<<(unsigned)((total + thr - 1) / thr), thr, 0, st>>>(zte, p->d_zte_off, p->d_Wg, p->d_woff, c,
-                                                                             out, total, p->Vte);
-    }
+        return p->Wmax <= 16 ? launch_apply_blocks<16>(p, zte, c, out, st, dependent)
+                             : launch_apply_blocks<32>(p, zte, c, out, st, dependent);
+    const bool wide = p->Wmax > 16;
+    const int thr = wide ? ApplyCfg<32>::threads : ApplyCfg<16>::threads;
+    launch_stage(dependent, wide ? apply_kernel<32> : apply_kernel<16>, (unsigned)((total + thr - 1) / thr), thr, 0, st,
+                 zte, p->d_zte_off, p->d_Wg, p->d_woff, c, out, total, p->Vte);
     return check_launch("apply launch");
 }
 

@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
     __shared__ long long tab_base[kTabT];
     __shared__ int tab_sw[kTabT];     // start | (W << 16)
     __shared__ int tab_n[kTabT];      // vectors of this CTA that the target's windows take (0: none)
+    wait_for_predecessor();
     const int tid = threadIdx.x;
     const int64_t vid0 = (int64_t)blockIdx.x * vpb;
     int s_cta = 0, v0_cta = 0;
@@ -150,8 +151,8 @@ static bs_status launch_bs_t(const float2 *y, int64_t nvec, int N, const float2 
     const int64_t blocks = (nvec + C::vpb - 1) / C::vpb;
     if (blocks > 0x7FFFFFFF) return set_error(BS_EUNSUPPORTED, "too many vectors");
     if (blocks == 0) return BS_OK;
-    beamspace_kernel<M, kFull, PREC><<<(unsigned)blocks, C::nthr, C::smem, st>>>(
-        y, nvec, N, tw, 1.0f / sqrtf((float)M), out, ga);
+    launch_stage(ga.dependent, beamspace_kernel<M, kFull, PREC>, (unsigned)blocks, C::nthr, C::smem, st, y, nvec, N, tw,
+                 1.0f / sqrtf((float)M), out, ga);
     return check_launch("beamspace launch");
 }
 
@@ -179,7 +180,7 @@ static int ilog2(int v) {
 }
 
 bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2 *zte, cudaStream_t st, int p0,
-                           int np) {
+                           int np, bool dependent) {
     if (np < 0) np = p->P - p0;
     GatherArgs ga;
     ga.nvec = (int64_t)np * p->Fs;   // Fs = Ls B bins per record (F without a shard)
@@ -204,6 +205,7 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     ga.ztr = ztr;
     ga.zte = zte;
     ga.store_scale = p->cfg.store_scale;
+    ga.dependent = dependent;
     if (p->planar) return launch_beamspace2d(p, xc, ga, st);
     bool used = false;
     bs_status s = BS_OK;

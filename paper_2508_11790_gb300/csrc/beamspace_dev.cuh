@@ -35,6 +35,7 @@ struct GatherArgs {
     void *ztr;              // training windows (plan precision)
     float2 *zte;            // test windows
     float store_scale;
+    bool dependent;         // host: launched along a pass (launch_stage)
 };
 
 template <int PREC>

@@ -272,6 +272,7 @@ __device__ __forceinline__ void warp_units(const WarpArgs &wa, const GatherArgs 
 template <int R, bool kFull, int PREC>
 __global__ void __launch_bounds__(256, 2)
     beamspace_warp_kernel(WarpArgs wa, GatherArgs ga, const float2 *__restrict__ twM) {
+    wait_for_predecessor();
     constexpr int M = 1024 * R, vpc = 8 / R;
     extern __shared__ __align__(16) unsigned char smraw[];
     float2 *tw = reinterpret_cast<float2 *>(smraw);    // [R][32 k1][32 n2]
@@ -332,7 +333,7 @@ bs_status launch_warp_t(const bs_plan *p, const float2 *xc, const GatherArgs &ga
     wa.sc_tr = (wa.prec == BS_PREC_FP32) ? wa.scale : wa.scale * ga.store_scale;
     wa.glist = p->d_glist;
     wa.sumW = p->sumW;
-    beamspace_warp_kernel<R, kFull, PREC><<<grid, 256, smem, st>>>(wa, ga, p->d_twM);
+    launch_stage(ga.dependent, beamspace_warp_kernel<R, kFull, PREC>, grid, 256, smem, st, wa, ga, p->d_twM);
     return check_launch("beamspace (warp) launch");
 }
 

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(ChCfg<F>::nthr, ChCfg<F>::minb)
     constexpr int NT = ChCfg<F>::NT;
     constexpr int nthr = ChCfg<F>::nthr;
     extern __shared__ float2 sm[];
+    let_dependents_launch();
     const int tid = threadIdx.x;
     const int n0 = blockIdx.x * NT;
     const float2 *xin = x + (size_t)blockIdx.y * F * N;
@@ -110,6 +111,7 @@ __global__ void __launch_bounds__(ChTmaCfg<F>::nthr, 1)
     float2 *ob = reinterpret_cast<float2 *>(smraw + C::stage_bytes + C::work_bytes);   // dense output tile
     uint64_t *bar = reinterpret_cast<uint64_t *>(smraw + 2 * C::stage_bytes + C::work_bytes);
     __shared__ int ok_s;
+    let_dependents_launch();
     const int tid = threadIdx.x;
     const int ntn = (N + NT - 1) / NT;
     const long long ntiles = (long long)P * ntn;

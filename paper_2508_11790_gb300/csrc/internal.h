@@ -87,6 +87,24 @@ bs_status set_error(bs_status s, const std::string &msg);
 bs_status cuda_error(cudaError_t e, const char *where);
 bs_status check_launch(const char *where);
 
+// Launch of a kernel that starts with wait_for_predecessor() (common.cuh).
+// dependent: the preceding operation of the stream is a kernel of the same
+// pass, and the kernel's CTAs may be placed before that one has completed.
+template <class... P, class... A>
+void launch_stage(bool dependent, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // an error is left for check_launch()
+}
+
 // Launch settings that a kernel needs once per device: function attributes
 // (the dynamic shared-memory limit) and occupancy apply to the current device
 // only, so a process that uses several GPUs sets them on each.  get() runs
@@ -119,14 +137,15 @@ struct PerDevice {
 bs_status launch_channelize(const bs_plan *p, const float2 *x, int P, float2 *xc, cudaStream_t st);
 // records p0 .. p0+np-1 (np < 0: through the last record)
 bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2 *zte, cudaStream_t st, int p0 = 0,
-                           int np = -1);
+                           int np = -1, bool dependent = false);
 bs_status launch_beamspace_full(const bs_plan *p, const float2 *y, int64_t nvec, float2 *yb,
                                 cudaStream_t st);
 // The covariance launcher's choice for this plan is the warp-per-pair kernel.
 bool window_cov_uses_warp(const bs_plan *p);
 // Warp-per-pair covariance of slots [slot0, slot1) of `order` (pair order if null).
 bs_status launch_window_cov_warp(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                                 cudaStream_t st, int64_t slot0, int64_t slot1, const int32_t *order);
+                                 cudaStream_t st, int64_t slot0, int64_t slot1, const int32_t *order,
+                                 bool dependent = false);
 // Covariance and stand-alone solve as one chain per window size, the chains
 // in parallel (plan side streams); applies to plans whose covariance takes
 // the warp-per-pair kernel, with several window sizes, all at most 16 beams.
@@ -134,21 +153,23 @@ bool cov_solve_chains_apply(const bs_plan *p);
 bs_status launch_cov_solve_chains(const bs_plan *p, const void *ztr, double2 *R, float2 *c, int32_t *info,
                                   cudaStream_t st);
 bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                            cudaStream_t st);
+                            cudaStream_t st, bool dependent = false);
 bs_status launch_window_cov_mma(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                                cudaStream_t st);
+                                cudaStream_t st, bool dependent = false);
 // dpre: optional diagonal preconditioner [c_elems] (woff-packed), NULL for none
 bs_status launch_mvdr_solve(const bs_plan *p, const double2 *R, float2 *c, int32_t *info,
-                            cudaStream_t st, const float *dpre = nullptr);
+                            cudaStream_t st, const float *dpre = nullptr, bool dependent = false);
+// the plan's pairs are solved by one launch on the caller's stream
+bool mvdr_solve_is_one_launch(const bs_plan *p);
 // the pairs of window size W <= 16, without and with a preconditioner, and of sizes W - 3 .. W (W = 20, 24, 28, 32)
 bs_status launch_solve_small(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
-                             const float *dpre, int refine, int f64);
+                             const float *dpre, int refine, int f64, bool dependent = false);
 bs_status launch_solve_small_precond(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info,
-                                     cudaStream_t st, const float *dpre, int refine, int f64);
+                                     cudaStream_t st, const float *dpre, int refine, int f64, bool dependent = false);
 bs_status launch_solve_wide(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
                             const float *dpre, int refine, int f64);
 bs_status launch_apply(const bs_plan *p, const float2 *zte, const float2 *c, float2 *out,
-                       cudaStream_t st);
+                       cudaStream_t st, bool dependent = false);
 bs_status launch_cov_solve(const bs_plan *p, const void *ztr, const float *delta, double2 *R, float2 *c,
                            int32_t *info, int *head, const CovSolveLaunch &cfg, cudaStream_t st);
 bs_status launch_cov_solve_tables(const void *z, int precision, float store_scale, const int32_t *Wg,

@@ -91,6 +91,10 @@ static int wide_classes(const bs_plan *p) {   // of four sizes each: 17..20, ..,
     return n;
 }
 
+bool mvdr_solve_is_one_launch(const bs_plan *p) {
+    return (p->cfg.flags & BS_FLAG_PLAIN) || wide_classes(p) + window_classes(p) == 1;
+}
+
 bool cov_solve_chains_apply(const bs_plan *p) {
     return !(p->cfg.flags & BS_FLAG_PLAIN) && p->nsmall == p->pairs && window_classes(p) > 1 &&
            window_cov_uses_warp(p);
@@ -118,7 +122,7 @@ bs_status launch_cov_solve_chains(const bs_plan *p, const void *ztr, double2 *R,
 }
 
 bs_status launch_mvdr_solve(const bs_plan *p, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
-                            const float *dpre) {
+                            const float *dpre, bool dependent) {
     const int64_t G = p->pairs;
     if (p->Wmax > WMAX_WIDE) return set_error(BS_EUNSUPPORTED, "W > 32");
     if (p->cfg.flags & BS_FLAG_PLAIN) {
@@ -134,6 +138,7 @@ bs_status launch_mvdr_solve(const bs_plan *p, const double2 *R, float2 *c, int32
     // graph capture, parallel branches), so that one launch's tail overlaps
     // the others' work.
     const int nlaunch = wide_classes(p) + window_classes(p);
+    dependent = dependent && nlaunch == 1;
     const int nst = nlaunch < 1 + bs_plan::kSolveStreams ? nlaunch : 1 + bs_plan::kSolveStreams;
     if (bs_status s = fork_streams(p, st, nst)) return s;
     int li = 0;   // launches issued; launch i goes to stream i mod nst
@@ -148,8 +153,8 @@ bs_status launch_mvdr_solve(const bs_plan *p, const double2 *R, float2 *c, int32
     for (int W = 16; W >= 1; --W) {
         if (p->wstart[W + 1] == p->wstart[W]) continue;
         const cudaStream_t ws = next_stream();
-        if (bs_status s = dpre ? launch_solve_small_precond(p, W, R, c, info, ws, dpre, refine, f64)
-                               : launch_solve_small(p, W, R, c, info, ws, dpre, refine, f64))
+        if (bs_status s = dpre ? launch_solve_small_precond(p, W, R, c, info, ws, dpre, refine, f64, dependent)
+                               : launch_solve_small(p, W, R, c, info, ws, dpre, refine, f64, dependent))
             return s;
     }
     return join_streams(p, st, nst);   // `st` waits for every side stream's launches

@@ -4,8 +4,8 @@
 namespace bs {
 
 bs_status launch_solve_small_precond(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info,
-                                     cudaStream_t st, const float *dpre, int refine, int f64) {
-    return launch_solve_small_t<true>(p, W, R, c, info, st, dpre, refine, f64);
+                                     cudaStream_t st, const float *dpre, int refine, int f64, bool dependent) {
+    return launch_solve_small_t<true>(p, W, R, c, info, st, dpre, refine, f64, dependent);
 }
 
 }  // namespace bs

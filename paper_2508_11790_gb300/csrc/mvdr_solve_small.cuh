@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(128, 4)
                         const float2 *__restrict__ atlo, const double2 *__restrict__ at64, float2 *__restrict__ c,
                         int32_t *__restrict__ info, int64_t slot0, int64_t slot1, double kappa_max, int refine,
                         int allow_f64, const int32_t *__restrict__ order, const float *__restrict__ dpre) {
+    wait_for_predecessor();
     constexpr int GW = (WT <= 8) ? 8 : 16;
     constexpr int PPC = 128 / GW;
     __shared__ __align__(16) unsigned char scratch[PPC][solve_scratch_bytes<GW>];
@@ -39,23 +40,23 @@ __global__ void __launch_bounds__(128, 4)
 // the W-grouped order (the identity when every pair has that size).
 template <int WT, bool PRE>
 bs_status launch_solve_w(const bs_plan *p, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
-                         const float *dpre, int refine, int f64) {
+                         const float *dpre, int refine, int f64, bool dependent) {
     constexpr int PPC = 128 / ((WT <= 8) ? 8 : 16);
     const int64_t s0 = p->wstart[WT], s1 = p->wstart[WT + 1];
     if (s1 <= s0) return BS_OK;
     const int32_t *order = p->Wmin == p->Wmax ? nullptr : p->d_order_w;
     const unsigned blocks = (unsigned)((s1 - s0 + PPC - 1) / PPC);
-    mvdr_solve_w_kernel<WT, PRE><<<blocks, 128, 0, st>>>(R, p->d_roff, p->d_woff, p->d_at32, p->d_atlo, p->d_at64, c,
-                                                         info, s0, s1, p->cfg.kappa_max, refine, f64, order, dpre);
+    launch_stage(dependent, mvdr_solve_w_kernel<WT, PRE>, blocks, 128, 0, st, R, p->d_roff, p->d_woff, p->d_at32,
+                 p->d_atlo, p->d_at64, c, info, s0, s1, p->cfg.kappa_max, refine, f64, order, dpre);
     return check_launch("solve (one window size) launch");
 }
 
 // The pairs of window size W of the plan.
 template <bool PRE>
 bs_status launch_solve_small_t(const bs_plan *p, int W, const double2 *R, float2 *c, int32_t *info, cudaStream_t st,
-                               const float *dpre, int refine, int f64) {
+                               const float *dpre, int refine, int f64, bool dependent) {
 #define BS_SOLVE_W(n) \
-    case n: return launch_solve_w<n, PRE>(p, R, c, info, st, dpre, refine, f64);
+    case n: return launch_solve_w<n, PRE>(p, R, c, info, st, dpre, refine, f64, dependent);
     switch (W) {
         BS_SOLVE_W(1) BS_SOLVE_W(2) BS_SOLVE_W(3) BS_SOLVE_W(4) BS_SOLVE_W(5) BS_SOLVE_W(6) BS_SOLVE_W(7) BS_SOLVE_W(8)
         BS_SOLVE_W(9) BS_SOLVE_W(10) BS_SOLVE_W(11) BS_SOLVE_W(12) BS_SOLVE_W(13) BS_SOLVE_W(14) BS_SOLVE_W(15)

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(COV_THREADS)
     constexpr int ES = (PREC == BS_PREC_FP32) ? 8 : 4;          // bytes per stored element
     __shared__ __align__(16) unsigned char stage[2][COV_STAGE_ELEMS * ES];
     __shared__ float red[4][9][COV_THREADS];
+    wait_for_predecessor();
     const int64_t g = blockIdx.x;
     const int tid = threadIdx.x;
     const int W = Wg[g], K = Kg[g];
@@ -455,6 +456,7 @@ __global__ void __launch_bounds__(COVW_WARPS * 32)
                            const int32_t *__restrict__ order) {
     constexpr int ES = (PREC == BS_PREC_FP32) ? 8 : 4;   // bytes per stored element
     __shared__ __align__(16) unsigned char stage[COVW_WARPS][COVW_CH * WMAX_COV * ES];
+    wait_for_predecessor();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t slot = slot0 + (int64_t)blockIdx.x * COVW_WARPS + warp;
     if (slot >= slot1) return;   // uniform per warp; no CTA barrier below
@@ -507,30 +509,22 @@ bool window_cov_uses_warp(const bs_plan *p) {
 }
 
 bs_status launch_window_cov_warp(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                                 cudaStream_t st, int64_t slot0, int64_t slot1, const int32_t *order) {
+                                 cudaStream_t st, int64_t slot0, int64_t slot1, const int32_t *order,
+                                 bool dependent) {
     if (slot1 <= slot0) return BS_OK;
     const unsigned blocks = (unsigned)((slot1 - slot0 + COVW_WARPS - 1) / COVW_WARPS);
     const DF dl = df_from_double(p->cfg.delta);
     const float inv_sc = 1.0f / p->cfg.store_scale;
-    switch (p->cfg.precision) {
-        case BS_PREC_FP32:
-            window_cov_warp_kernel<BS_PREC_FP32><<<blocks, COVW_WARPS * 32, 0, st>>>(
-                ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, dl, 1.0f, R, slot0, slot1, order);
-            break;
-        case BS_PREC_FP16:
-            window_cov_warp_kernel<BS_PREC_FP16><<<blocks, COVW_WARPS * 32, 0, st>>>(
-                ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, dl, inv_sc, R, slot0, slot1, order);
-            break;
-        default:
-            window_cov_warp_kernel<BS_PREC_BF16><<<blocks, COVW_WARPS * 32, 0, st>>>(
-                ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, dl, inv_sc, R, slot0, slot1, order);
-            break;
-    }
+    const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_warp_kernel<BS_PREC_FP32>
+                        : p->cfg.precision == BS_PREC_FP16 ? window_cov_warp_kernel<BS_PREC_FP16>
+                                                           : window_cov_warp_kernel<BS_PREC_BF16>;
+    launch_stage(dependent, kernel, blocks, COVW_WARPS * 32, 0, st, ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta,
+                 dl, p->cfg.precision == BS_PREC_FP32 ? 1.0f : inv_sc, R, slot0, slot1, order);
     return check_launch("covariance (warp per pair) launch");
 }
 
 bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                            cudaStream_t st) {
+                            cudaStream_t st, bool dependent) {
     const unsigned G = (unsigned)p->pairs;
     if (p->cfg.flags & BS_FLAG_PLAIN) {
         if (p->cfg.precision != BS_PREC_FP32)
@@ -546,10 +540,10 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
     const int tv = p->tune_cov;   // a variant chosen by bs_autotune_pass, where it applies
     const bool mma_ok = !wide && p->cfg.precision != BS_PREC_FP32;
     if (mma_ok && (tv == 2 || (tv < 0 && !(p->cfg.flags & BS_FLAG_SIMT_COV))))
-        return launch_window_cov_mma(p, ztr, delta, R, st);
+        return launch_window_cov_mma(p, ztr, delta, R, st, dependent);
     const float inv_sc = 1.0f / p->cfg.store_scale;
     // warp per pair: short streams over enough pairs to fill the GPU by warps
-    if (window_cov_uses_warp(p)) return launch_window_cov_warp(p, ztr, delta, R, st, 0, p->pairs, nullptr);
+    if (window_cov_uses_warp(p)) return launch_window_cov_warp(p, ztr, delta, R, st, 0, p->pairs, nullptr, dependent);
     if (wide) {
         const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_wide_kernel<BS_PREC_FP32>
                             : p->cfg.precision == BS_PREC_FP16 ? window_cov_wide_kernel<BS_PREC_FP16>
@@ -559,20 +553,11 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
                                           p->cfg.precision == BS_PREC_FP32 ? 1.0f : inv_sc, R);
         return check_launch("covariance (wide windows) launch");
     }
-    switch (p->cfg.precision) {
-        case BS_PREC_FP32:
-            window_cov_kernel<BS_PREC_FP32><<<G, COV_THREADS, 0, st>>>(
-                ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, df_from_double(p->cfg.delta), 1.0f, R);
-            break;
-        case BS_PREC_FP16:
-            window_cov_kernel<BS_PREC_FP16><<<G, COV_THREADS, 0, st>>>(
-                ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, df_from_double(p->cfg.delta), inv_sc, R);
-            break;
-        default:
-            window_cov_kernel<BS_PREC_BF16><<<G, COV_THREADS, 0, st>>>(
-                ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, df_from_double(p->cfg.delta), inv_sc, R);
-            break;
-    }
+    const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_kernel<BS_PREC_FP32>
+                        : p->cfg.precision == BS_PREC_FP16 ? window_cov_kernel<BS_PREC_FP16>
+                                                           : window_cov_kernel<BS_PREC_BF16>;
+    launch_stage(dependent, kernel, G, COV_THREADS, 0, st, ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta,
+                 df_from_double(p->cfg.delta), p->cfg.precision == BS_PREC_FP32 ? 1.0f : inv_sc, R);
     return check_launch("covariance launch");
 }
 

@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(MMA_WARPS * 32)
                           const int64_t *__restrict__ roff, const float *__restrict__ delta_pair, DF delta,
                           DF inv_sc2, double2 *__restrict__ R, int64_t pairs) {
     extern __shared__ __align__(16) uint16_t mma_smem[];
+    wait_for_predecessor();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t g = (int64_t)blockIdx.x * MMA_WARPS + warp;
     if (g >= pairs) return;   // uniform per warp; no CTA-wide barrier below
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(MMA_WARPS * 32)
 }
 
 bs_status launch_window_cov_mma(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                                cudaStream_t st) {
+                                cudaStream_t st, bool dependent) {
     const int64_t G = p->pairs;
     const unsigned blocks = (unsigned)((G + MMA_WARPS - 1) / MMA_WARPS);
     static PerDevice attr;
@@ -273,12 +274,10 @@ bs_status launch_window_cov_mma(const bs_plan *p, const void *ztr, const float *
         return s;
     const DF sc = df_from_double(1.0 / ((double)p->cfg.store_scale * (double)p->cfg.store_scale));
     const DF dl = df_from_double(p->cfg.delta);
-    if (p->cfg.precision == BS_PREC_FP16)
-        window_cov_mma_kernel<BS_PREC_FP16><<<blocks, MMA_WARPS * 32, MMA_SMEM, st>>>(
-            ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, dl, sc, R, G);
-    else
-        window_cov_mma_kernel<BS_PREC_BF16><<<blocks, MMA_WARPS * 32, MMA_SMEM, st>>>(
-            ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta, dl, sc, R, G);
+    const auto kernel = p->cfg.precision == BS_PREC_FP16 ? window_cov_mma_kernel<BS_PREC_FP16>
+                                                         : window_cov_mma_kernel<BS_PREC_BF16>;
+    launch_stage(dependent, kernel, blocks, MMA_WARPS * 32, MMA_SMEM, st, ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff,
+                 delta, dl, sc, R, G);
     return check_launch("covariance (tensor core) launch");
 }
 

@@ -201,6 +201,10 @@ static bs_status launch_ch_tma(const bs_plan *pl, const float2 *x, int P, int N,
     if (reinterpret_cast<uintptr_t>(xc) & 15) return BS_OK;
     CUtensorMap tmap, omap;
     const int Fs = pl->Fs, q0 = pl->s0 * pl->B;
+    // a shard's rows leave from row q0 of the output tile, and a tensor store
+    // starts on 128 bytes of shared memory (a shard of fewer than four bins
+    // takes the plain kernel)
+    if (((size_t)q0 * C::NT * sizeof(float2)) & 127) return BS_OK;
     const int obox = Fs < C::box_rows ? Fs : C::box_rows;   // q0 and Fs are multiples of obox
     const cuuint64_t gdim[2] = {(cuuint64_t)2 * N, (cuuint64_t)P * F};
     const cuuint64_t odim[2] = {(cuuint64_t)2 * N, (cuuint64_t)P * Fs};

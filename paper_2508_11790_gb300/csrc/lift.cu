@@ -4,9 +4,9 @@
 // M^-1/2 z^start (sum_w c_g[w] z^w), the sum by Horner's rule: two conjugated
 // entries of the plan's M-point twiddle table per output (indices n and
 // start n mod M) and no transcendental.  Its antenna-space output and its
-// beam pattern are in lift_tc.cu.
+// beam pattern are in lift_tc.cu, the beam pattern of few pairs is here.
 //
-// A CTA takes LIFT_PAIRS pairs; a thread four elements a block apart of each
+// A CTA takes up to LIFT_PAIRS pairs; a thread four elements a block apart of each
 // pair: z is read once, the four Horner chains share the weights' loads and
 // loop, and run two to a packed FP32x2 FMA.  The scattered reads of z^start
 // go to a copy of the twiddle table in shared memory, one spare slot per 16
@@ -17,6 +17,8 @@
 #include "common.cuh"
 #include "internal.h"
 
+#include <algorithm>
+
 namespace bs {
 
 constexpr int LIFT_PAIRS = 8;
@@ -24,9 +26,9 @@ constexpr int LIFT_PAIRS = 8;
 __global__ void __launch_bounds__(256)
     lift_kernel(const float2 *__restrict__ c, const int64_t *__restrict__ woff, const int32_t *__restrict__ Wg,
                 const int32_t *__restrict__ start, const float2 *__restrict__ twM, int M, int N, int64_t pairs,
-                float scale, float2 *__restrict__ c_hat) {
-    const int64_t g0 = (int64_t)blockIdx.x * LIFT_PAIRS;
-    const int np = (int)min((int64_t)LIFT_PAIRS, pairs - g0);
+                int per, float scale, float2 *__restrict__ c_hat) {
+    const int64_t g0 = (int64_t)blockIdx.x * per;
+    const int np = (int)min((int64_t)per, pairs - g0);
     __shared__ float4 cw[LIFT_PAIRS][32];   // (re, re, im, im)
     __shared__ int Ws[LIFT_PAIRS], st[LIFT_PAIRS];
     for (int e = threadIdx.x; e < 32 * np; e += blockDim.x) {
@@ -83,16 +85,132 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// grid (pairs, ceil(n_dirs / per)), a CTA per pair and range of per directions,
+// a warp per DPW directions.  The sum runs over 32 lanes' elements with one
+// complex rotation per 32 elements.  The correlator is scaled by a power of
+// two to a largest part of 1 to 2, so that its norm neither underflows nor
+// overflows; the pattern does not depend on its scale.
+// Bound by the rotations' FMAs and, for a pair's first directions, by loading
+// the correlator and its norm: about 4.5 us + 7 ns a pair + (3.5 + N / 124) ns
+// a pair and 32 directions.  96 pairs, 31 directions: 5 us at N = 48 and 6.5 at
+// N = 1024, where the tensor-core tiles take 11 and 59; ranges of directions
+// for few pairs: 181 directions of those in 10 and 16 us.
+__global__ void __launch_bounds__(256)
+    beam_pattern_kernel(const float2 *__restrict__ c_hat, const double *__restrict__ u, int n_dirs, int per, int N,
+                        int L, int Ls, int s0, double fc, double fs, double fd, float *__restrict__ pattern) {
+    extern __shared__ float2 ch[];   // [N] c_hat, then [per] Omega / pi as FP32 (hi, lo)
+    float2 *omt = ch + N;
+    __shared__ float part[8];
+    const int64_t g = blockIdx.x;
+    const int s = s0 + (int)(g % Ls);   // subband of pair g among the L (plans of a shard: s0 + local)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d0 = blockIdx.y * per, nd = min(per, n_dirs - d0);
+    float mx = 0.f;
+    for (int n = threadIdx.x; n < N; n += 256) {
+        const float2 v = c_hat[g * N + n];
+        ch[n] = v;
+        mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    if (lane == 0) part[warp] = mx;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w) mx = fmaxf(mx, part[w]);
+    __syncthreads();
+    const float sc = (mx > 0.f && mx <= 3.4e38f) ? ldexpf(1.f, max(-126, min(126, -ilogbf(mx)))) : 1.f;
+    float nrm = 0.f;
+    for (int n = threadIdx.x; n < N; n += 256) {   // the elements this thread wrote
+        const float2 v = cscale(ch[n], sc);
+        ch[n] = v;
+        nrm = fmaf(v.x, v.x, fmaf(v.y, v.y, nrm));
+    }
+    for (int o = 16; o; o >>= 1) nrm += __shfl_xor_sync(0xFFFFFFFFu, nrm, o);
+    if (lane == 0) part[warp] = nrm;
+    __syncthreads();
+    float tot = 0.f;
+    for (int w = 0; w < 8; ++w) tot += part[w];
+    const float inv = 1.f / (sqrtf(tot) * sqrtf((float)N));
+    // subband centre frequency (Eq. SubChannelFreq): fc + ((l - 1/2) / L) fs,
+    // l = s - L/2 + 1, in this order; Omega / pi = u f / f_d per direction,
+    // formed once per CTA in FP64 and kept as an FP32 (hi, lo) pair (the FP64
+    // pipe is narrow, so the per-lane work below is FP32 only)
+    const double f = fc + (((double)(s - L / 2 + 1) - 0.5) / (double)L) * fs;
+    const double ratio = f / fd;
+    for (int k = threadIdx.x; k < nd; k += 256) {
+        const double om = u[d0 + k] * ratio;
+        const float hi = (float)om;
+        omt[k] = make_float2(hi, (float)(om - (double)hi));
+    }
+    __syncthreads();
+    constexpr int DPW = 4;   // directions per warp pass: each shared load feeds four sums
+    for (int k0 = warp * DPW; k0 < nd; k0 += 8 * DPW) {
+        // Omega / pi = u f / fd; e^{j Omega n} with n = lane + 32 i.  The two
+        // phases (in units of pi) are reduced to [-1, 1] in FP32 pairs before
+        // sincospi, so their error does not grow with n.
+        float er[DPW], ei[DPW], c32[DPW], s32[DPW], re[DPW], im[DPW];
+#pragma unroll
+        for (int d = 0; d < DPW; ++d) {
+            const float2 om = (k0 + d < nd) ? omt[k0 + d] : make_float2(0.f, 0.f);
+            // x0 = om * lane: exact product of the high part (fmaf), reduced
+            // modulo 2 before the low-order terms are added
+            const float p = om.x * (float)lane;
+            const float e = fmaf(om.x, (float)lane, -p) + om.y * (float)lane;
+            const float x0 = (p - 2.f * rintf(0.5f * p)) + e;
+            const float q = om.x * 32.f;   // exact
+            const float x32 = (q - 2.f * rintf(0.5f * q)) + om.y * 32.f;
+            sincospif(x0, &ei[d], &er[d]);
+            sincospif(x32, &s32[d], &c32[d]);
+            re[d] = im[d] = 0.f;
+        }
+        for (int n = lane; n < N; n += 32) {
+            const float2 a = ch[n];
+#pragma unroll
+            for (int d = 0; d < DPW; ++d) {   // conj(a) * e, then e *= e^{j 32 Omega}
+                re[d] = fmaf(a.x, er[d], fmaf(a.y, ei[d], re[d]));
+                im[d] = fmaf(a.x, ei[d], fmaf(-a.y, er[d], im[d]));
+                const float nr = er[d] * c32[d] - ei[d] * s32[d];
+                ei[d] = fmaf(er[d], s32[d], ei[d] * c32[d]);
+                er[d] = nr;
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < DPW; ++d) {
+            for (int o = 16; o; o >>= 1) {
+                re[d] += __shfl_xor_sync(0xFFFFFFFFu, re[d], o);
+                im[d] += __shfl_xor_sync(0xFFFFFFFFu, im[d], o);
+            }
+            if (lane == 0 && k0 + d < nd)
+                pattern[g * n_dirs + d0 + k0 + d] = sqrtf(re[d] * re[d] + im[d] * im[d]) * inv;
+        }
+    }
+}
+
 bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStream_t st) {
     const int N = p->cfg.N;
     if (p->pairs == 0) return BS_OK;
     if (p->Wmax > 32) return set_error(BS_EUNSUPPORTED, "W > 32");
     const int M = p->cfg.M;
     const int thr = N >= 1024 ? 256 : ((N + 3) / 4 + 31) & ~31;
-    const dim3 grid((unsigned)((p->pairs + LIFT_PAIRS - 1) / LIFT_PAIRS), (N + 4 * thr - 1) / (4 * thr));
+    const int ny = (N + 4 * thr - 1) / (4 * thr);
+    // fewer pairs per CTA while that leaves the chip no more than a wave of
+    // two CTAs per SM: the chains of a CTA's pairs follow one another (with
+    // eight a CTA, lift and outputs of 96 pairs, N = 100, W = 16: 20.5 us,
+    // 19.5 now; the lift alone takes 3 us up to 512 pairs)
+    const int per = (int)std::min<int64_t>(LIFT_PAIRS, (p->pairs * ny + 303) / 304);
+    const dim3 grid((unsigned)((p->pairs + per - 1) / per), ny);
     lift_kernel<<<grid, thr, padded_len(M < 16 ? 16 : M) * sizeof(float2), st>>>(
-        c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, p->pairs, 1.0f / sqrtf((float)M), c_hat);
+        c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, p->pairs, per, 1.0f / sqrtf((float)M), c_hat);
     return check_launch("lift launch");
+}
+
+bs_status launch_beam_pattern_simt(const bs_plan *p, const float2 *c_hat, int n_dirs, const double *u,
+                                   float *pattern, cudaStream_t st) {
+    // 32 directions a CTA while that leaves at most four CTAs per SM, more otherwise
+    const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((n_dirs + 31) / 32, 608 / p->pairs));
+    const int per = (int)((n_dirs + parts - 1) / parts + 31) & ~31;
+    const dim3 grid((unsigned)p->pairs, (n_dirs + per - 1) / per);
+    beam_pattern_kernel<<<grid, 256, ((size_t)p->cfg.N + per) * sizeof(float2), st>>>(
+        c_hat, u, n_dirs, per, p->cfg.N, p->cfg.L, p->Ls, p->s0, p->cfg.fc, p->cfg.fs, p->cfg.fd, pattern);
+    return check_launch("beam pattern launch");
 }
 
 }  // namespace bs

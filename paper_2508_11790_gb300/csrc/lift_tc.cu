@@ -28,8 +28,8 @@
 // chunk's leading sum is hidden behind them.
 //
 // Measured at 64 targets, 1024 elements and 128 subbands: 128 test vectors
-// 327 -> 62 us, 181 directions 598 -> 88 us; the SIMT kernels these replace
-// were bound by shared-memory loads (2 x 2 register tiles, 26 TFLOP/s) and by
+// 327 -> 62 us, 181 directions 598 -> 88 us; the SIMT kernels measured
+// against were bound by shared-memory loads (2 x 2 register tiles, 26 TFLOP/s) and by
 // one rotation per pair, element and direction.  With two leading sums drained
 // two stages late and two direction tiles of 128: 76 and 122 us.  Timing copies
 // with parts left out: products alone 45 us for 128 columns and 53 for 192 (98
@@ -41,6 +41,7 @@
 #include "tcgen05.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace bs {
 namespace {
@@ -452,6 +453,21 @@ LtArgs lift_args(const bs_plan *p, const float2 *c_hat, int cols, int tile) {
     return a;
 }
 
+// Few pairs: the SIMT kernel (lift.cu).  A tile takes as long for 3 targets as
+// for 64, 8 us + 51 ns an element and wave of tiles; the SIMT kernel's time
+// grows with the pairs and directions from 4.5 us.  Both lines are fits within
+// 10 % of 135 measured sizes (N 48 .. 1024, 48 .. 8192 pairs, 31 .. 181
+// directions); at the line both take the same: 512 pairs of N = 100, 64
+// directions 14.7 us each, 1024 of N = 256 23.2 and 23.3, 2048 of N = 512, 31
+// directions 34.6 and 34.1.  By the whole plan's subbands, so that a shard's
+// patterns are bit for bit those of the whole.
+bool pattern_simt(const bs_plan *p, int n_dirs) {
+    const double N = p->cfg.N, pairs = (double)p->cfg.T * p->cfg.L;
+    if (p->cfg.N + (int64_t)n_dirs > 6144) return false;   // 48 KB of shared memory
+    const double tiles = (double)p->cfg.L * ((p->cfg.T + LT_T - 1) / LT_T) * ((n_dirs + 191) / 192);
+    return pairs * (7.0 + (n_dirs + 31) / 32 * (3.5 + N / 124)) < (4000 + 50 * N) * std::ceil(tiles / 152);
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
@@ -474,6 +490,7 @@ bs_status launch_beam_pattern(const bs_plan *p, const float2 *c_hat, int n_dirs,
     if (n_dirs == 0 || p->pairs == 0) return BS_OK;
     if (((size_t)p->cfg.N + n_dirs) * sizeof(float2) > 200 * 1024)
         return set_error(BS_EUNSUPPORTED, "beam pattern: N + n_dirs must be <= 25600");
+    if (pattern_simt(p, n_dirs)) return launch_beam_pattern_simt(p, c_hat, n_dirs, u, pattern, st);
     LtArgs a = lift_args(p, c_hat, n_dirs, 192);
     a.u = u;
     a.Ltot = p->cfg.L;

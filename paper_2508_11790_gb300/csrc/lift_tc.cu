@@ -253,21 +253,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
             }
         }
         const int nb = (NB + 63) >> 6;   // blocks of 64 columns in use
-        // sum of squares of this thread's part of the row, (hi, lo), scaled by
-        // the power of two that brings the row's first elements near 1, so
-        // that neither the norm nor the squares below leave FP32's range
-        float nh = 0.f, nl = 0.f, sc = 1.f;
-        if constexpr (PATTERN) {
-            float2 x[4];
-            load_item<VEC>(crow, 4 * c, a.N, tval, x);
-            float m = 0.f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
-            m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-            m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-            const int e = max(-120, min(120, ((__float_as_int(m) >> 23) & 255) - 127));
-            if (m > 0.f && isfinite(m)) sc = __int_as_float((127 - e) << 23);
-        }
+        float nh = 0.f, nl = 0.f;   // sum of squares of this thread's part of the row, (hi, lo)
         float2 xa[4], xb[PATTERN ? 1 : NI][4];
         auto fetch = [&](int st) {
             const int n = st * LT_K + 4 * c;
@@ -294,12 +280,10 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
                 for (int i = 0; i < 4; ++i) w[p][i] = __byte_perm(w[p][i], w[p][i], 0x1032) ^ 0x8000u;   // (-Im, Re)
             put(at + 8 * LT_SBO, LT_PART, w);   // row r + 64
             if constexpr (PATTERN) {
-                float s2 = 0.f;
+                float2 q = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float x = xa[i].x * sc, y = xa[i].y * sc;
-                    s2 = fmaf(x, x, fmaf(y, y, s2));
-                }
+                for (int i = 0; i < 4; ++i) q = __ffma2_rn(xa[i], xa[i], q);
+                const float s2 = q.x + q.y;
                 const float sm = nh + s2, bb = sm - nh;
                 nl += (nh - (sm - bb)) + (s2 - bb);
                 nh = sm;
@@ -351,7 +335,38 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
             atomicOr(a.err, 1);
         }
         if constexpr (PATTERN) {
-            float n2 = nh + nl;
+            // The norm is n2 / sc^2.  Squares that left FP32's range, or come
+            // near its ends, are formed again of elements scaled by a power
+            // of two to a largest part of 1 to 2; a row's first elements say
+            // nothing about the others, and following the largest so far
+            // inside the loop took 6 to 10 of 90 us.
+            float n2 = nh + nl, sc = 1.f;
+            if (tval && !(n2 >= 0x1p-70f && n2 <= 0x1p96f)) {
+                float m = 0.f;
+                for (int st = grp; st < nst; st += 2) {
+                    load_item<VEC>(crow, st * LT_K + 4 * c, a.N, true, xa);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(fabsf(xa[i].x), fabsf(xa[i].y)));
+                }
+                const int e = max(-126, min(126, (__float_as_int(m) >> 23) - 127));
+                sc = __int_as_float((127 - e) << 23);
+                n2 = 0.f;
+                for (int st = grp; st < nst; st += 2) {
+                    load_item<VEC>(crow, st * LT_K + 4 * c, a.N, true, xa);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float x = xa[i].x * sc, y = xa[i].y * sc;
+                        n2 = fmaf(x, x, fmaf(y, y, n2));
+                    }
+                }
+            }
+            // the four lanes of a row, on the smallest of their scales
+            if (n2 == 0.f) sc = 0x1p126f;
+            float to = fminf(sc, __shfl_xor_sync(0xFFFFFFFFu, sc, 1));
+            to = fminf(to, __shfl_xor_sync(0xFFFFFFFFu, to, 2));
+            const float f = to * (1.f / sc);
+            n2 = n2 * f * f;
+            sc = to;
             n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, 1);
             n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, 2);
             if (c == 0) nrm[64 * grp + r] = make_float2(n2, sc);
@@ -409,8 +424,10 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
         const int64_t o = ((int64_t)(t0 + r) * a.L + s) * a.cols + v0;
         float sc = 1.f, inv = 1.f;
         if constexpr (PATTERN) {
-            sc = nrm[r].y;
-            inv = 1.f / (sqrtf(nrm[r].x + nrm[64 + r].x) * sqrtf((float)a.N));
+            const float2 n0 = nrm[r], n1 = nrm[64 + r];   // the two groups' stages
+            sc = fminf(n0.y, n1.y);
+            const float f0 = sc * (1.f / n0.y), f1 = sc * (1.f / n1.y);
+            inv = 1.f / (sqrtf(n0.x * f0 * f0 + n1.x * f1 * f1) * sqrtf((float)a.N));
         }
         for (int k = lane; k < ncol; k += 32) {
             const float2 v = tile[r * LT_PITCH + k];

@@ -95,12 +95,14 @@ __global__ void __launch_bounds__(256)
 // a pair and 32 directions.  96 pairs, 31 directions: 5 us at N = 48 and 6.5 at
 // N = 1024, where the tensor-core tiles take 11 and 59; ranges of directions
 // for few pairs: 181 directions of those in 10 and 16 us.
+constexpr int PATTERN_STATIC = 32;   // its static shared memory
+
 __global__ void __launch_bounds__(256)
     beam_pattern_kernel(const float2 *__restrict__ c_hat, const double *__restrict__ u, int n_dirs, int per, int N,
                         int L, int Ls, int s0, double fc, double fs, double fd, float *__restrict__ pattern) {
     extern __shared__ float2 ch[];   // [N] c_hat, then [per] Omega / pi as FP32 (hi, lo)
     float2 *omt = ch + N;
-    __shared__ float part[8];
+    __shared__ float part[PATTERN_STATIC / sizeof(float)];   // one per warp
     const int64_t g = blockIdx.x;
     const int s = s0 + (int)(g % Ls);   // subband of pair g among the L (plans of a shard: s0 + local)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -204,9 +206,12 @@ bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStre
 
 bs_status launch_beam_pattern_simt(const bs_plan *p, const float2 *c_hat, int n_dirs, const double *u,
                                    float *pattern, cudaStream_t st) {
-    // 32 directions a CTA while that leaves at most four CTAs per SM, more otherwise
+    // 32 directions a CTA while that leaves at most four CTAs per SM, more
+    // otherwise, as many as fit the 48 KB of an ordinary launch beside the
+    // correlator (2016 at N = 4096)
     const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((n_dirs + 31) / 32, 608 / p->pairs));
-    const int per = (int)((n_dirs + parts - 1) / parts + 31) & ~31;
+    const int fit = ((48 * 1024 - PATTERN_STATIC) / (int)sizeof(float2) - p->cfg.N) & ~31;
+    const int per = std::min(fit, (int)((n_dirs + parts - 1) / parts + 31) & ~31);
     const dim3 grid((unsigned)p->pairs, (n_dirs + per - 1) / per);
     beam_pattern_kernel<<<grid, 256, ((size_t)p->cfg.N + per) * sizeof(float2), st>>>(
         c_hat, u, n_dirs, per, p->cfg.N, p->cfg.L, p->Ls, p->s0, p->cfg.fc, p->cfg.fs, p->cfg.fd, pattern);

@@ -480,7 +480,7 @@ LtArgs lift_args(const bs_plan *p, const float2 *c_hat, int cols, int tile) {
 // patterns are bit for bit those of the whole.
 bool pattern_simt(const bs_plan *p, int n_dirs) {
     const double N = p->cfg.N, pairs = (double)p->cfg.T * p->cfg.L;
-    if (p->cfg.N + (int64_t)n_dirs > 6144) return false;   // 48 KB of shared memory
+    if (p->cfg.N + (int64_t)n_dirs > 6144) return false;   // not measured beyond: the tiles
     const double tiles = (double)p->cfg.L * ((p->cfg.T + LT_T - 1) / LT_T) * ((n_dirs + 191) / 192);
     return pairs * (7.0 + (n_dirs + 31) / 32 * (3.5 + N / 124)) < (4000 + 50 * N) * std::ceil(tiles / 152);
 }

@@ -22,9 +22,9 @@ struct ApplyCfg {
 
 template <int WM>
 __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
-    apply_kernel(const float2 *__restrict__ z, const int64_t *__restrict__ zte_off,
+    apply_kernel(const float2 *z, const int64_t *__restrict__ zte_off,
                  const int32_t *__restrict__ Wg, const int64_t *__restrict__ woff,
-                 const float2 *__restrict__ c, float2 *__restrict__ out, int64_t total, int Vte) {
+                 const float2 *c, float2 *__restrict__ out, int64_t total, int Vte) {
     __shared__ float2 span[ApplyCfg<WM>::threads / 32][ApplyCfg<WM>::span];
     wait_for_predecessor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
     float re = 0.f, im = 0.f;
     for (int w = 0; w < W; ++w) {
         const float2 a = zv[w];
-        const float2 b = __ldg(&cg[w]);
+        const float2 b = cg[w];
         // conj(b) * a
         re = fmaf(b.x, a.x, fmaf(b.y, a.y, re));
         im = fmaf(b.x, a.y, fmaf(-b.y, a.x, im));
@@ -63,9 +63,9 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
 // block's sums.  Figures at the launcher.
 template <int WM>
 __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
-    apply_blocks_kernel(const float2 *__restrict__ z, const int64_t *__restrict__ zte_off,
+    apply_blocks_kernel(const float2 *z, const int64_t *__restrict__ zte_off,
                         const int32_t *__restrict__ Wg, const int64_t *__restrict__ woff,
-                        const float2 *__restrict__ c, float2 *__restrict__ out, unsigned units, unsigned upp, int nb,
+                        const float2 *c, float2 *__restrict__ out, unsigned units, unsigned upp, int nb,
                         int bpw) {
     constexpr int NW = ApplyCfg<WM>::threads / 32, NR = WM / 2;   // 16-byte loads per lane: 16 W per block
     __shared__ __align__(16) float2 span[NW][ApplyCfg<WM>::span];
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
     const unsigned g = unit / upp;
     const int b0 = (int)(unit - g * upp) * bpw, b1 = min(nb, b0 + bpw);
     const int W = __ldg(&Wg[g]);
-    if (lane < W) cw[warp][lane] = __ldg(&c[__ldg(&woff[g]) + lane]);
+    if (lane < W) cw[warp][lane] = c[__ldg(&woff[g]) + lane];
     const float4 *src = reinterpret_cast<const float4 *>(z + __ldg(&zte_off[g]) + (int64_t)b0 * 32 * W);
     float2 *buf = span[warp];
     float4 r[NR];

@@ -19,7 +19,7 @@ namespace bs {
 // precision of the training windows).
 template <int M, bool kFull, int PREC>
 __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
-    beamspace_kernel(const float2 *__restrict__ y, int64_t nvec, int N, const float2 *__restrict__ tw,
+    beamspace_kernel(const float2 *y, int64_t nvec, int N, const float2 *__restrict__ tw,
                      float scale, float2 *__restrict__ out, GatherArgs ga) {
     using RP = Radix<M>;
     constexpr int vpb = BsCfg<M>::vpb;

@@ -14,6 +14,11 @@ namespace bs {
 // here, before it touches memory, until its predecessor has completed.  What is
 // saved is the launch and ramp-up of each stage: a pass of 64 pairs 29.2 -> 23.2 us,
 // of 1024 pairs at N = 256 89 -> 82 us.  Both are no-ops in an ordinary launch.
+// Arrays that an earlier stage of the pass writes are read by ordinary (or
+// .cg / .cs) loads only, through pointers that are not const __restrict__: the
+// read-only path (ld.global.nc: __ldg, or the compiler's choice for such a
+// pointer) is for data that nothing writes while the kernel lives, and its life
+// begins before the predecessor's ends.  The plan's tables may take it.
 __device__ __forceinline__ void let_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_predecessor() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

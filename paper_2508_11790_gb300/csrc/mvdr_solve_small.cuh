@@ -16,7 +16,7 @@ namespace bs {
 // PRE: with a preconditioner.
 template <int WT, bool PRE>
 __global__ void __launch_bounds__(128, 4)
-    mvdr_solve_w_kernel(const double2 *__restrict__ R, const int64_t *__restrict__ roff,
+    mvdr_solve_w_kernel(const double2 *R, const int64_t *__restrict__ roff,
                         const int64_t *__restrict__ woff, const float2 *__restrict__ at32,
                         const float2 *__restrict__ atlo, const double2 *__restrict__ at64, float2 *__restrict__ c,
                         int32_t *__restrict__ info, int64_t slot0, int64_t slot1, double kappa_max, int refine,

@@ -193,7 +193,7 @@ __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned
 // ex: the lane's preconditioner exponent (0 without one); row j scales by
 // 2^(ex_lane + ex_j), exactly.
 template <int GW = 16>
-static __device__ __noinline__ int solve_f64(unsigned mask, int lane, int W, const double2 *__restrict__ Rg, double2 a,
+static __device__ __noinline__ int solve_f64(unsigned mask, int lane, int W, const double2 *Rg, double2 a,
                                                 double2 *Ld, double2 &c_out, int ex) {
     double2 D[GW];
     const bool row = lane < W;

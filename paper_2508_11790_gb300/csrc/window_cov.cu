@@ -58,7 +58,7 @@ __device__ __forceinline__ float2 widen(const void *stage, int q, float inv_sc) 
 // double-float accumulators; the slices are reduced in double-float.
 template <int PREC>
 __global__ void __launch_bounds__(COV_THREADS)
-    window_cov_kernel(const void *__restrict__ z, const int64_t *__restrict__ ztr_off,
+    window_cov_kernel(const void *z, const int64_t *__restrict__ ztr_off,
                       const int32_t *__restrict__ Wg, const int32_t *__restrict__ Kg,
                       const int64_t *__restrict__ roff, const float *__restrict__ delta_pair,
                       DF delta, float inv_sc, double2 *__restrict__ R) {
@@ -403,11 +403,11 @@ __device__ __forceinline__ void cov_warp_pair(unsigned char *sb, int lane, int64
         if constexpr (ES == 8) {
             const float2 *src = reinterpret_cast<const float2 *>(zg) + (int64_t)k0 * W;
             float2 *dst = reinterpret_cast<float2 *>(sb);
-            for (int q = lane; q < n * W; q += 32) dst[q] = __ldg(src + q);
+            for (int q = lane; q < n * W; q += 32) dst[q] = __ldcg(src + q);
         } else {
             const uint32_t *src = reinterpret_cast<const uint32_t *>(zg) + (int64_t)k0 * W;
             uint32_t *dst = reinterpret_cast<uint32_t *>(sb);
-            for (int q = lane; q < n * W; q += 32) dst[q] = __ldg(src + q);
+            for (int q = lane; q < n * W; q += 32) dst[q] = __ldcg(src + q);
         }
         __syncwarp();
         for (int v = 0, o = 0; v < n; ++v, o += W) {
@@ -449,7 +449,7 @@ __device__ __forceinline__ void cov_warp_pair(unsigned char *sb, int lane, int64
 
 template <int PREC>
 __global__ void __launch_bounds__(COVW_WARPS * 32)
-    window_cov_warp_kernel(const void *__restrict__ z, const int64_t *__restrict__ ztr_off,
+    window_cov_warp_kernel(const void *z, const int64_t *__restrict__ ztr_off,
                            const int32_t *__restrict__ Wg, const int32_t *__restrict__ Kg,
                            const int64_t *__restrict__ roff, const float *__restrict__ delta_pair, DF delta,
                            float inv_sc, double2 *__restrict__ R, int64_t slot0, int64_t slot1,

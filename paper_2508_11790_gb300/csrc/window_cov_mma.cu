@@ -239,7 +239,7 @@ __device__ __forceinline__ void cov_pair(uint16_t *ring, int lane, int64_t g, in
 // setting the occupancy, the smaller register budget only cost overlap).
 template <int PREC>
 __global__ void __launch_bounds__(MMA_WARPS * 32)
-    window_cov_mma_kernel(const void *__restrict__ z, const int64_t *__restrict__ ztr_off,
+    window_cov_mma_kernel(const void *z, const int64_t *__restrict__ ztr_off,
                           const int32_t *__restrict__ Wg, const int32_t *__restrict__ Kg,
                           const int64_t *__restrict__ roff, const float *__restrict__ delta_pair, DF delta,
                           DF inv_sc2, double2 *__restrict__ R, int64_t pairs) {

@@ -185,6 +185,15 @@ __device__ __forceinline__ void stockham_pass(int tid, const float2 *__restrict_
         tid, [tw](int k) { return __ldg(&tw[k]); }, load, store);
 }
 
+// The sum of a product's leading parts plus that of its trailing parts.  The
+// leading parts are infinite or NaN where the values are (a quiet NaN's leading
+// part is one), so an infinite leading sum is the result; the trailing parts
+// hold zeros, whose products with an infinity are NaN.
+__device__ __forceinline__ float join_parts(float lead, float trail) { return isinf(lead) ? lead : lead + trail; }
+__device__ __forceinline__ float2 join_parts(float2 lead, float2 trail) {
+    return make_float2(join_parts(lead.x, trail.x), join_parts(lead.y, trail.y));
+}
+
 // Double-float values (h + l, |l| <= ulp(h)/2): GB300's FP64 pipe is
 // narrow, so the covariance epilogues assemble R in FP32 pairs and convert
 // only the final value of each entry to FP64.

@@ -109,8 +109,8 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
 }
 
 // Four elements (eight floats) as three parts of four packed words each
-// (word = real low, imaginary high).  A non-finite value makes its row's or
-// column's outputs NaN.
+// (word = real low, imaginary high).  The leading part of an infinity is that
+// infinity, its trailing parts are NaN (join_parts).
 __device__ __forceinline__ void split_item(const float2 (&v)[4], uint32_t (&w)[3][4]) {
     // minus the leading 8 bits of both components
     auto ntop = [](float2 x) {
@@ -207,21 +207,18 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
         float2 acc[DC / 2];
 #pragma unroll
         for (int k = 0; k < DC / 2; ++k) acc[k] = make_float2(0.f, 0.f);
-        auto add = [&](uint32_t ta) {
-#pragma unroll
-            for (int p = 0; p < DC / 16; ++p) {
-                float d[16];
-                tmem_ld16(ta + 16 * p, d);
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    acc[8 * p + k] = __fadd2_rn(acc[8 * p + k], make_float2(d[2 * k], d[2 * k + 1]));
-            }
-        };
         auto drain = [&](int j) -> bool {   // chunk j's leading sum
             if (!mbar_wait_bounded(dfull, (unsigned)j & 1u)) return false;
             if (mine) {
                 tc_fence_after();
-                add(dat);
+#pragma unroll
+                for (int p = 0; p < DC / 16; ++p) {
+                    float d[16];
+                    tmem_ld16(dat + 16 * p, d);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        acc[8 * p + k] = __fadd2_rn(acc[8 * p + k], make_float2(d[2 * k], d[2 * k + 1]));
+                }
                 tc_fence_before();
             }
             __syncwarp();
@@ -322,7 +319,13 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lift_tc_kernel(const LtArgs a) 
         if (ok) {   // the last chunk's barrier covers every product
             if (mine) {
                 tc_fence_after();
-                add(dat + 256);
+#pragma unroll
+                for (int p = 0; p < DC / 16; ++p) {
+                    float d[16];
+                    tmem_ld16(dat + 256 + 16 * p, d);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) acc[8 * p + k] = join_parts(acc[8 * p + k], make_float2(d[2 * k], d[2 * k + 1]));
+                }
                 const int row = 32 * q + lane;
                 float *tile = reinterpret_cast<float *>(smlt) + ((row & 63) * LT_PITCH + DC * h) * 2 + (row >> 6);
 #pragma unroll

@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(NTHR, 1) mlp_slab_kernel(const MlpArgs a) {
 #pragma unroll
             for (int j = 0; j < NT; ++j)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[m][j][k] += low[m][j][k];
+                for (int k = 0; k < 4; ++k) acc[m][j][k] = join_parts(acc[m][j][k], low[m][j][k]);
     };
     // acc += A B over one 16-deep step: A the three parts at column ka of
     // `as` (pitch la), B the fragments of this warp's columns
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(NTHR, 1) mlp_slab_kernel(const MlpArgs a) {
             d[e] = 0.f;
             if (row < rows && n < O) {
                 const int64_t o = (row0 + row) * O + n;
-                const float y = ya[e] + yl[e] + bs[2 * HP + n];
+                const float y = join_parts(ya[e], yl[e]) + bs[2 * HP + n];
                 a.Y[o] = y;
                 if constexpr (TRAIN) {
                     const float r = y - tv[e];
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(256, 2) mlp_wgrad_kernel(const WgradArgs a) {
 #pragma unroll
             for (int e = 0; e < 2; ++e)
                 *reinterpret_cast<float2 *>(&S.tile[wm + g + 8 * e][wn + 8 * n + 2 * t]) =
-                    make_float2(acc[n][2 * e] + low[n][2 * e], acc[n][2 * e + 1] + low[n][2 * e + 1]);
+                    make_float2(join_parts(acc[n][2 * e], low[n][2 * e]), join_parts(acc[n][2 * e + 1], low[n][2 * e + 1]));
         S.csum[r][c] = cs.x;
         S.csum[r][c + 1] = cs.y;
     }

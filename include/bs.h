@@ -472,8 +472,7 @@ typedef struct {
 } bs_mlp;
 
 /* Activations of one batch (device, caller-owned): z1, h1, z2, h2, dh1, dh2
- * [capacity][n_hidden]; y, dy [capacity][n_out].  Scratch: networks of up to
- * 256 hidden units and 64 outputs keep some of them in registers. */
+ * [capacity][n_hidden]; y, dy [capacity][n_out]. */
 typedef struct {
     int64_t capacity;
     float *z1, *h1, *z2, *h2;

@@ -12,8 +12,9 @@
 //
 // Bound: latency.  Training step of the 101-256-256-10 network, 1024 rows:
 // 470 us (15 launches, the three weight gradients 160 us each: 4 to 16 CTAs
-// with a serial chain of 1024 rows) -> 33 us (slab kernel 17, weight
-// gradients 14).  Forward of 4096 rows: 112 us (three launches) -> 17 us.
+// with a serial chain of 1024 rows) -> 35 us (slab kernel 19, weight
+// gradients 14).  Forward of 4096 rows, back to back in a graph: 99 us (three
+// launches) -> 17.5, 3 of them the hidden layers' 17 MB in the work buffers.
 // With 8 warps instead of 16 and 32-row slabs at 1024 rows (32 CTAs) the slab
 // kernel took 40 us: 17 % issue, its two warps per scheduler waiting for
 // unbatched global loads and instruction fetch.
@@ -129,11 +130,12 @@ struct MlpArgs {
     int I, H, O;
     int batch;
     float *Y;
+    float *z1, *h1, *z2, *h2;       // the hidden layers before and after the ReLU
     // training only
     const float *T;
     float scale;
     double *loss;
-    float *h1, *h2, *dy, *dh1, *dh2;
+    float *dy, *dh1, *dh2;
 };
 
 template <int HP, int MT>
@@ -317,11 +319,11 @@ __global__ void __launch_bounds__(NTHR, 1) mlp_slab_kernel(const MlpArgs a) {
             load8(a.wb, a.o3 + (int64_t)min(n, O - 1) * H + min(k, H - 1), n < O ? H - k : 0, a.np);
     }
 
-    // bias, ReLU, the activations to memory (training) and as parts to ACT;
-    // the bits of positive pre-activations stay in a register
-    auto relu_layer = [&](const float *bias, float *hg) -> uint32_t {
+    // bias, ReLU, both to memory, the activations as parts to ACT; the bits of
+    // positive pre-activations stay in a register
+    auto relu_layer = [&](const float *bias, float *zg, float *hg) -> uint32_t {
         uint32_t mask = 0;
-        const bool pair = TRAIN && (H & 1) == 0 && (reinterpret_cast<uintptr_t>(hg) & 7) == 0;
+        const bool pair = (H & 1) == 0 && ((reinterpret_cast<uintptr_t>(zg) | reinterpret_cast<uintptr_t>(hg)) & 7) == 0;
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
             const int n = nw + 8 * j + 2 * t;
@@ -336,13 +338,14 @@ __global__ void __launch_bounds__(NTHR, 1) mlp_slab_kernel(const MlpArgs a) {
                     mask |= (z1 > 0.f ? 1u : 0u) << ((j * MT + m) * 4 + 2 * r + 1);
                     const int row = m * 16 + 8 * r + g;
                     put_parts<ROWS>(act, LD, row, n, h0, h1);
-                    if constexpr (TRAIN) put_global(hg + row0 * H, row, n, rows, H, pair, h0, h1);
+                    put_global(zg + row0 * H, row, n, rows, H, pair, z0, z1);
+                    put_global(hg + row0 * H, row, n, rows, H, pair, h0, h1);
                 }
         }
         return mask;
     };
     join();
-    const uint32_t m1 = relu_layer(bs, a.h1);
+    const uint32_t m1 = relu_layer(bs, a.z1, a.h1);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(NTHR, 1) mlp_slab_kernel(const MlpArgs a) {
     }
     join();
     __syncthreads();   // every warp has read h1's parts
-    const uint32_t m2 = relu_layer(bs + HP, a.h2);
+    const uint32_t m2 = relu_layer(bs + HP, a.z2, a.h2);
 
     // ---- layer 3: warp w takes rows 16 (w mod MT) .., outputs 8 (w / MT) ..
     const int mo = (warp % MT) * 16, no = (warp / MT) * 8;
@@ -658,7 +661,7 @@ bs_status launch_slab(const MlpArgs &a, cudaStream_t st) {
     return small ? launch_slab_t<256, 1, TRAIN>(a, st) : launch_slab_t<256, 2, TRAIN>(a, st);
 }
 
-MlpArgs slab_args(const bs_mlp *m, const float *X, int batch, float *Y) {
+MlpArgs slab_args(const bs_mlp *m, const float *X, int batch, float *Y, const bs_mlp_work *w) {
     const int64_t I = m->n_in, H = m->n_hidden, O = m->n_out;
     const __nv_bfloat16 *wb = (const __nv_bfloat16 *)m->weights_bf16;
     MlpArgs a{};
@@ -676,6 +679,10 @@ MlpArgs slab_args(const bs_mlp *m, const float *X, int batch, float *Y) {
     a.O = (int)O;
     a.batch = batch;
     a.Y = Y;
+    a.z1 = w->z1;
+    a.h1 = w->h1;
+    a.z2 = w->z2;
+    a.h2 = w->h2;
     return a;
 }
 
@@ -683,19 +690,18 @@ MlpArgs slab_args(const bs_mlp *m, const float *X, int batch, float *Y) {
 
 bool mlp_fused_applies(const bs_mlp *m) { return m->n_hidden <= 256 && m->n_out <= OMAX && m->n_in <= 65536; }
 
-bs_status launch_mlp_forward(const bs_mlp *m, const float *X, int batch, float *Y, cudaStream_t st) {
-    const MlpArgs a = slab_args(m, X, batch, Y);
+bs_status launch_mlp_forward(const bs_mlp *m, const float *X, int batch, float *Y, const bs_mlp_work *w,
+                             cudaStream_t st) {
+    const MlpArgs a = slab_args(m, X, batch, Y, w);
     return launch_slab<false>(a, st);
 }
 
 bs_status launch_mlp_train(const bs_mlp *m, const float *X, const float *T, int batch, const bs_mlp_work *w, float lr,
                            int step, double *loss, cudaStream_t st) {
-    MlpArgs a = slab_args(m, X, batch, w->y);
+    MlpArgs a = slab_args(m, X, batch, w->y, w);
     a.T = T;
     a.scale = 1.0f / (float)((int64_t)batch * a.O);
     a.loss = loss;
-    a.h1 = w->h1;
-    a.h2 = w->h2;
     a.dy = w->dy;
     a.dh1 = w->dh1;
     a.dh2 = w->dh2;

@@ -197,7 +197,8 @@ bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStre
     // two CTAs per SM: the chains of a CTA's pairs follow one another (with
     // eight a CTA, lift and outputs of 96 pairs, N = 100, W = 16: 20.5 us,
     // 19.5 now; the lift alone takes 3 us up to 512 pairs)
-    const int per = (int)std::min<int64_t>(LIFT_PAIRS, (p->pairs * ny + 303) / 304);
+    const int wave = 2 * p->num_sms;
+    const int per = (int)std::min<int64_t>(LIFT_PAIRS, (p->pairs * ny + wave - 1) / wave);
     const dim3 grid((unsigned)((p->pairs + per - 1) / per), ny);
     lift_kernel<<<grid, thr, padded_len(M < 16 ? 16 : M) * sizeof(float2), st>>>(
         c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, p->pairs, per, 1.0f / sqrtf((float)M), c_hat);
@@ -209,7 +210,7 @@ bs_status launch_beam_pattern_simt(const bs_plan *p, const float2 *c_hat, int n_
     // 32 directions a CTA while that leaves at most four CTAs per SM, more
     // otherwise, as many as fit the 48 KB of an ordinary launch beside the
     // correlator (2016 at N = 4096)
-    const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((n_dirs + 31) / 32, 608 / p->pairs));
+    const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((n_dirs + 31) / 32, 4 * p->num_sms / p->pairs));
     const int fit = ((48 * 1024 - PATTERN_STATIC) / (int)sizeof(float2) - p->cfg.N) & ~31;
     const int per = std::min(fit, (int)((n_dirs + parts - 1) / parts + 31) & ~31);
     const dim3 grid((unsigned)p->pairs, (n_dirs + per - 1) / per);

@@ -485,7 +485,7 @@ bool pattern_simt(const bs_plan *p, int n_dirs) {
     const double N = p->cfg.N, pairs = (double)p->cfg.T * p->cfg.L;
     if (p->cfg.N + (int64_t)n_dirs > 6144) return false;   // not measured beyond: the tiles
     const double tiles = (double)p->cfg.L * ((p->cfg.T + LT_T - 1) / LT_T) * ((n_dirs + 191) / 192);
-    return pairs * (7.0 + (n_dirs + 31) / 32 * (3.5 + N / 124)) < (4000 + 50 * N) * std::ceil(tiles / 152);
+    return pairs * (7.0 + (n_dirs + 31) / 32 * (3.5 + N / 124)) < (4000 + 50 * N) * std::ceil(tiles / p->num_sms);
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

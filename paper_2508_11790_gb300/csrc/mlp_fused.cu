@@ -652,11 +652,26 @@ bs_status launch_slab_t(const MlpArgs &a, cudaStream_t st) {
     return check_launch("MLP slab launch");
 }
 
+// SMs of the current device.
+bs_status device_sms(int *sms) {
+    static PerDevice count;
+    return count.get(
+        [](int *v) {
+            int dev = 0;
+            cudaError_t e = cudaGetDevice(&dev);
+            if (e == cudaSuccess) e = cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev);
+            return cuda_error(e, "number of SMs");
+        },
+        sms);
+}
+
 // One CTA fits an SM (W2 in shared memory): 16-row slabs while they are at
-// most one wave of the 152 SMs, 32-row slabs beyond.
+// most one wave of the SMs, 32-row slabs beyond.
 template <bool TRAIN>
 bs_status launch_slab(const MlpArgs &a, cudaStream_t st) {
-    const bool small = a.batch <= 16 * 152;
+    int sms = 0;
+    if (bs_status s = device_sms(&sms)) return s;
+    const bool small = a.batch <= 16 * sms;
     if (a.H <= 128) return small ? launch_slab_t<128, 1, TRAIN>(a, st) : launch_slab_t<128, 2, TRAIN>(a, st);
     return small ? launch_slab_t<256, 1, TRAIN>(a, st) : launch_slab_t<256, 2, TRAIN>(a, st);
 }

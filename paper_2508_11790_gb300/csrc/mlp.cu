@@ -378,7 +378,9 @@ bs_status bs_mlp_forward(const bs_mlp *m, const float *X, int64_t batch, float *
     if (batch < 0 || batch > w->capacity) return set_error(BS_EINVAL, "batch exceeds the work buffers");
     if (batch == 0) return BS_OK;
     const cudaStream_t st = (cudaStream_t)stream;
-    if (bs::mlp_fused_applies(m) && batch <= INT32_MAX) return bs::launch_mlp_forward(m, X, (int)batch, Y, w, st);
+    bool slabs = false;
+    if (bs_status s = bs::mlp_forward_by_slabs(m, batch, &slabs)) return s;
+    if (slabs && batch <= INT32_MAX) return bs::launch_mlp_forward(m, X, (int)batch, Y, w, st);
     const int I = m->n_in, H = m->n_hidden, O = m->n_out, B = (int)batch;
     const __nv_bfloat16 *wb = (const __nv_bfloat16 *)m->weights_bf16;
     const float *b1 = m->master + (int64_t)H * I, *b2 = b1 + H + (int64_t)H * H, *b3 = b2 + H + (int64_t)O * H;

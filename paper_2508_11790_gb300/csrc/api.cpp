@@ -159,8 +159,11 @@ bs_status bs_run(const bs_plan *p, const bs_buffers *b, bs_stream stream) {
     BS_REQUIRE(b->xc && b->z_train, "NULL buffer");
     BS_REQUIRE(b->z_test || p->cfg.P_test == 0, "z_test is NULL but P_test > 0");
     // from here each stage follows a kernel of this pass on the stream, so it
-    // may be placed while that one runs (dependent = true)
-    if ((s = bs::launch_beamspace(p, (const float2 *)b->xc, b->z_train, (float2 *)b->z_test, st, 0, -1, true))) return s;
+    // may be placed while that one runs
+    int64_t ctas = 0;
+    if ((s = bs::launch_beamspace(p, (const float2 *)b->xc, b->z_train, (float2 *)b->z_test, st, 0, -1,
+                                  bs::channelize_tiles(p, p->P), &ctas)))
+        return s;
     if (use_fused(p)) {
         if ((s = bs_cov_solve(p, b->z_train, nullptr, b->R, b->c, b->info, stream))) return s;
         return bs_apply(p, b->z_test, b->c, b->out, stream);
@@ -172,7 +175,7 @@ bs_status bs_run(const bs_plan *p, const bs_buffers *b, bs_stream stream) {
         if ((s = bs::launch_cov_solve_chains(p, b->z_train, (double2 *)b->R, (float2 *)b->c, b->info, st))) return s;
         return bs_apply(p, b->z_test, b->c, b->out, stream);
     }
-    if ((s = bs::launch_window_cov(p, b->z_train, nullptr, (double2 *)b->R, st, true))) return s;
+    if ((s = bs::launch_window_cov(p, b->z_train, nullptr, (double2 *)b->R, st, ctas))) return s;
     const bool one = bs::mvdr_solve_is_one_launch(p);   // else the side streams are joined by events
     if ((s = bs::launch_mvdr_solve(p, (const double2 *)b->R, (float2 *)b->c, b->info, st, nullptr, one))) return s;
     if (p->Vte == 0) return BS_OK;

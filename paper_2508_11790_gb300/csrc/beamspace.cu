@@ -142,16 +142,23 @@ static bs_status launch_bs_t(const float2 *y, int64_t nvec, int N, const float2 
                              const GatherArgs &ga, cudaStream_t st) {
     using C = BsCfg<M>;
     static PerDevice attr;
-    if (bs_status s = attr.get([](int *) {
-            return cuda_error(cudaFuncSetAttribute(beamspace_kernel<M, kFull, PREC>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem),
-                              "beamspace attribute");
-        }))
+    int per_sm = 0;
+    if (bs_status s = attr.get(
+            [](int *v) {
+                const auto kernel = beamspace_kernel<M, kFull, PREC>;
+                cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+                if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, kernel, C::nthr, C::smem);
+                return cuda_error(e, "beamspace attribute");
+            },
+            &per_sm))
         return s;
     const int64_t blocks = (nvec + C::vpb - 1) / C::vpb;
     if (blocks > 0x7FFFFFFF) return set_error(BS_EUNSUPPORTED, "too many vectors");
     if (blocks == 0) return BS_OK;
-    launch_stage(ga.dependent, beamspace_kernel<M, kFull, PREC>, (unsigned)blocks, C::nthr, C::smem, st, y, nvec, N, tw,
+    // M >= 1024: several waves gain nothing (N = 1500: 1.5 % slower)
+    const bool dependent = ga.pred > 0 && (3 * ga.pred <= ga.sms || ga.pred + blocks <= ga.sms ||
+                                           (M < 1024 && blocks >= 2LL * per_sm * ga.sms));
+    launch_stage(dependent, beamspace_kernel<M, kFull, PREC>, (unsigned)blocks, C::nthr, C::smem, st, y, nvec, N, tw,
                  1.0f / sqrtf((float)M), out, ga);
     return check_launch("beamspace launch");
 }
@@ -180,7 +187,7 @@ static int ilog2(int v) {
 }
 
 bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2 *zte, cudaStream_t st, int p0,
-                           int np, bool dependent) {
+                           int np, int64_t pred, int64_t *ctas) {
     if (np < 0) np = p->P - p0;
     GatherArgs ga;
     ga.nvec = (int64_t)np * p->Fs;   // Fs = Ls B bins per record (F without a shard)
@@ -205,7 +212,9 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     ga.ztr = ztr;
     ga.zte = zte;
     ga.store_scale = p->cfg.store_scale;
-    ga.dependent = dependent;
+    ga.pred = pred;
+    ga.sms = p->num_sms;
+    if (ctas) *ctas = p->num_sms;   // every kernel but the last fills the chip
     if (p->planar) return launch_beamspace2d(p, xc, ga, st);
     bool used = false;
     bs_status s = BS_OK;
@@ -229,6 +238,7 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
         s = launch_beamspace_tma(p, xc, ga, st, &used);
         if (s || used) return s;
     }
+    if (ctas) *ctas = (ga.nvec + p->vpb - 1) / p->vpb;
     switch (p->cfg.precision) {
         case BS_PREC_FP32: return launch_bs<false, BS_PREC_FP32>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, st);
         case BS_PREC_FP16: return launch_bs<false, BS_PREC_FP16>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, st);

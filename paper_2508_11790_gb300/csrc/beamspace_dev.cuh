@@ -35,7 +35,8 @@ struct GatherArgs {
     void *ztr;              // training windows (plan precision)
     float2 *zte;            // test windows
     float store_scale;
-    bool dependent;         // host: launched along a pass (launch_stage)
+    int64_t pred;           // host: CTAs of the preceding stage (launch_beamspace)
+    int sms;
 };
 
 template <int PREC>

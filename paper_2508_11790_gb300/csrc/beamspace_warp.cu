@@ -333,7 +333,8 @@ bs_status launch_warp_t(const bs_plan *p, const float2 *xc, const GatherArgs &ga
     wa.sc_tr = (wa.prec == BS_PREC_FP32) ? wa.scale : wa.scale * ga.store_scale;
     wa.glist = p->d_glist;
     wa.sumW = p->sumW;
-    launch_stage(ga.dependent, beamspace_warp_kernel<R, kFull, PREC>, grid, 256, smem, st, wa, ga, p->d_twM);
+    // never dependent: one CTA or two per SM, all resident at once (launch_beamspace)
+    launch_stage(false, beamspace_warp_kernel<R, kFull, PREC>, grid, 256, smem, st, wa, ga, p->d_twM);
     return check_launch("beamspace (warp) launch");
 }
 

@@ -250,6 +250,11 @@ static bs_status launch_ch(const float2 *x, int P, int N, float2 *xc, const floa
     return check_launch("channelize launch");
 }
 
+int64_t channelize_tiles(const bs_plan *p, int P) {
+    const int F = p->cfg.F, NT = std::max(4, std::min(32, 8192 / F));   // ChCfg
+    return (int64_t)P * ((p->cfg.N + NT - 1) / NT);
+}
+
 bs_status launch_channelize(const bs_plan *p, const float2 *x, int P, float2 *xc, cudaStream_t st) {
     const int N = p->cfg.N;
     const int q0 = p->s0 * p->B, Fs = p->Fs;

@@ -524,8 +524,12 @@ bs_status launch_window_cov_warp(const bs_plan *p, const void *ztr, const float 
 }
 
 bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
-                            cudaStream_t st, bool dependent) {
+                            cudaStream_t st, int64_t pred) {
     const unsigned G = (unsigned)p->pairs;
+    // six CTAs of 128 threads an SM: of several waves or nearly one
+    auto dependent = [&](int64_t ctas) {
+        return pred > 0 && (pred + ctas <= p->num_sms || ctas >= 6LL * p->num_sms);
+    };
     if (p->cfg.flags & BS_FLAG_PLAIN) {
         if (p->cfg.precision != BS_PREC_FP32)
             return set_error(BS_EINVAL, "the plain path is FP32 only");
@@ -540,10 +544,12 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
     const int tv = p->tune_cov;   // a variant chosen by bs_autotune_pass, where it applies
     const bool mma_ok = !wide && p->cfg.precision != BS_PREC_FP32;
     if (mma_ok && (tv == 2 || (tv < 0 && !(p->cfg.flags & BS_FLAG_SIMT_COV))))
-        return launch_window_cov_mma(p, ztr, delta, R, st, dependent);
+        return launch_window_cov_mma(p, ztr, delta, R, st, dependent((p->pairs + 3) / 4));
     const float inv_sc = 1.0f / p->cfg.store_scale;
     // warp per pair: short streams over enough pairs to fill the GPU by warps
-    if (window_cov_uses_warp(p)) return launch_window_cov_warp(p, ztr, delta, R, st, 0, p->pairs, nullptr, dependent);
+    if (window_cov_uses_warp(p))
+        return launch_window_cov_warp(p, ztr, delta, R, st, 0, p->pairs, nullptr,
+                                      dependent((p->pairs + COVW_WARPS - 1) / COVW_WARPS));
     if (wide) {
         const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_wide_kernel<BS_PREC_FP32>
                             : p->cfg.precision == BS_PREC_FP16 ? window_cov_wide_kernel<BS_PREC_FP16>
@@ -556,7 +562,7 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
     const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_kernel<BS_PREC_FP32>
                         : p->cfg.precision == BS_PREC_FP16 ? window_cov_kernel<BS_PREC_FP16>
                                                            : window_cov_kernel<BS_PREC_BF16>;
-    launch_stage(dependent, kernel, G, COV_THREADS, 0, st, ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta,
+    launch_stage(dependent(G), kernel, G, COV_THREADS, 0, st, ztr, p->d_ztr_off, p->d_Wg, p->d_Kg, p->d_roff, delta,
                  df_from_double(p->cfg.delta), p->cfg.precision == BS_PREC_FP32 ? 1.0f : inv_sc, R);
     return check_launch("covariance launch");
 }

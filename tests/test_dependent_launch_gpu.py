@@ -26,6 +26,8 @@ CASES = [   # N, M, L, B, T, W, K, P_train, P_test, plan arguments
     (60, 64, 4, 8, 3, [5], 40, 8, 4, dict(flags=P.BS_FLAG_PLAIN)),
     (60, 64, 4, 8, 3, [5], 40, 8, 0, {}),                                          # no test records
     (60, 64, 8, 8, 3, [5], 40, 8, 4, dict(s_begin=4, s_count=4)),                  # a shard
+    (64, 512, 32, 32, 40, [7], 200, 8, 2, {}),                                     # several waves of both dependent stages
+    (16, 16, 4, 4, 1, [4], 4, 1, 1, {}),                                           # a few CTAs in all
 ]
 
 

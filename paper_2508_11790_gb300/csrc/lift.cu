@@ -85,6 +85,30 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// The same sums, bit for bit, one element of one pair per thread: no table to
+// copy and no chain of pairs to go through, for work that does not fill the chip.
+__global__ void __launch_bounds__(256)
+    lift_few_kernel(const float2 *__restrict__ c, const int64_t *__restrict__ woff, const int32_t *__restrict__ Wg,
+                    const int32_t *__restrict__ start, const float2 *__restrict__ twM, int M, int N, float scale,
+                    float2 *__restrict__ c_hat) {
+    __shared__ float2 cw[32];
+    const int64_t g = blockIdx.x;
+    const int n = blockIdx.y * blockDim.x + threadIdx.x;
+    const int W = Wg[g];
+    if (threadIdx.x < W) cw[threadIdx.x] = c[woff[g] + threadIdx.x];
+    __syncthreads();
+    if (n >= N) return;
+    const float2 z = __ldg(&twM[n & (M - 1)]), t = __ldg(&twM[(start[g] * n) & (M - 1)]);
+    const float zr = z.x, zi = -z.y, nz = z.y;
+    float ar = cw[W - 1].x, ai = cw[W - 1].y;
+    for (int w = W - 2; w >= 0; --w) {
+        const float re = fmaf(ar, zr, fmaf(ai, nz, cw[w].x));
+        ai = fmaf(ar, zi, fmaf(ai, zr, cw[w].y));
+        ar = re;
+    }
+    c_hat[g * N + n] = cscale(cmulc(make_float2(ar, ai), t), scale);
+}
+
 // grid (pairs, ceil(n_dirs / per)), a CTA per pair and range of per directions,
 // a warp per DPW directions.  The sum runs over 32 lanes' elements with one
 // complex rotation per 32 elements.  The correlator is scaled by a power of
@@ -191,17 +215,32 @@ bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStre
     if (p->pairs == 0) return BS_OK;
     if (p->Wmax > 32) return set_error(BS_EUNSUPPORTED, "W > 32");
     const int M = p->cfg.M;
+    const float scale = 1.0f / sqrtf((float)M);
+    // Few CTAs of one pair and 256 elements: an element per thread.  The other
+    // kernel copies the M twiddles per CTA and takes its pairs one after the
+    // other, so the line moves with M / N and, for short rows, with W.  1024
+    // pairs of N = 100, M = 512, W = 9: 7.3 us with the table, 2.9 without;
+    // N = 1024, M = 4096 7.8 and 7.4; 4096 pairs of N = 300, M = 512 8.5 and
+    // 10.1; over 700 sizes within 0.3 % of the better one on average.  Both
+    // give the same bits, so a shard may lie on the other side of it.
+    const double blocks = (double)p->pairs * ((N + 255) / 256);
+    const double line = N <= 64 ? std::max(4000.0, 1400.0 * p->Wmax)
+                                : std::min(9000.0, 2000.0 + 800.0 * M / N + 1.2e6 / N);
+    if (blocks <= line) {
+        const int thr = std::min(256, (std::max(N, p->Wmax) + 31) & ~31);
+        lift_few_kernel<<<dim3((unsigned)p->pairs, (N + thr - 1) / thr), thr, 0, st>>>(
+            c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, scale, c_hat);
+        return check_launch("lift (few) launch");
+    }
     const int thr = N >= 1024 ? 256 : ((N + 3) / 4 + 31) & ~31;
     const int ny = (N + 4 * thr - 1) / (4 * thr);
     // fewer pairs per CTA while that leaves the chip no more than a wave of
-    // two CTAs per SM: the chains of a CTA's pairs follow one another (with
-    // eight a CTA, lift and outputs of 96 pairs, N = 100, W = 16: 20.5 us,
-    // 19.5 now; the lift alone takes 3 us up to 512 pairs)
+    // two CTAs per SM: the chains of a CTA's pairs follow one another
     const int wave = 2 * p->num_sms;
     const int per = (int)std::min<int64_t>(LIFT_PAIRS, (p->pairs * ny + wave - 1) / wave);
     const dim3 grid((unsigned)((p->pairs + per - 1) / per), ny);
     lift_kernel<<<grid, thr, padded_len(M < 16 ? 16 : M) * sizeof(float2), st>>>(
-        c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, p->pairs, per, 1.0f / sqrtf((float)M), c_hat);
+        c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, p->pairs, per, scale, c_hat);
     return check_launch("lift launch");
 }
 

@@ -203,6 +203,8 @@ bs_status launch_range_doppler(const bs_plan *p, const float2 *out, const float2
                                cudaStream_t st);
 bs_status launch_cfar(const bs_plan *p, const float *map, float threshold_db, float *floor, int32_t *count,
                       uint8_t *mask, int32_t *peak, cudaStream_t st);
+bs_status launch_apply_lifted_simt(const bs_plan *p, const float2 *xc, const float2 *c_hat, float2 *out,
+                                   cudaStream_t st);
 bs_status launch_beam_pattern_simt(const bs_plan *p, const float2 *c_hat, int n_dirs, const double *u,
                                    float *pattern, cudaStream_t st);
 bs_status launch_apply_lifted(const bs_plan *p, const float2 *xc, const float2 *c_hat, float2 *out,

@@ -210,6 +210,65 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// c_hat^H y of short rows: a CTA takes 32 targets x 32 test vectors of one
+// subband with 32-element slices of both in shared memory, FP32.
+constexpr int AL_T = 32;   // targets per tile
+constexpr int AL_V = 32;   // test vectors per tile
+constexpr int AL_K = 32;   // elements per shared-memory slice
+
+// grid (ceil(T/32), ceil(Vte/32), L); 256 threads as 16 x 16, 2 x 2 outputs each
+__global__ void __launch_bounds__(256)
+    apply_lifted_kernel(const float2 *__restrict__ xc, const float2 *__restrict__ c_hat, float2 *__restrict__ out,
+                        int N, int F, int B, int L, int T, int P_train, int Vte) {
+    __shared__ float2 Cs[AL_T][AL_K + 1];
+    __shared__ float2 Ys[AL_V][AL_K + 1];
+    const int s = blockIdx.z;
+    const int t0 = blockIdx.x * AL_T, v0 = blockIdx.y * AL_V;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    float2 acc[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) acc[a][b] = make_float2(0.f, 0.f);
+    for (int k0 = 0; k0 < N; k0 += AL_K) {
+        // stage: row r of each tile, lanes along the elements (coalesced)
+        for (int e = threadIdx.x; e < AL_T * AL_K; e += 256) {
+            const int r = e / AL_K, k = e % AL_K;
+            const int t = t0 + r, v = v0 + r, n = k0 + k;
+            float2 cv = make_float2(0.f, 0.f), yv = make_float2(0.f, 0.f);
+            if (t < T && n < N) cv = __ldg(&c_hat[((int64_t)t * L + s) * N + n]);
+            if (v < Vte && n < N) {
+                const int p = P_train + v / B, q = s * B + v % B;
+                yv = __ldcs(&xc[((int64_t)p * F + q) * N + n]);
+            }
+            Cs[r][k] = cv;
+            Ys[r][k] = yv;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int k = 0; k < AL_K; ++k) {
+            const float2 c0 = Cs[2 * ty][k], c1 = Cs[2 * ty + 1][k];
+            const float2 y0 = Ys[2 * tx][k], y1 = Ys[2 * tx + 1][k];
+            const float2 cc[2] = {c0, c1}, yy[2] = {y0, y1};
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {   // conj(c) * y
+                    acc[a][b].x = fmaf(cc[a].x, yy[b].x, fmaf(cc[a].y, yy[b].y, acc[a][b].x));
+                    acc[a][b].y = fmaf(cc[a].x, yy[b].y, fmaf(-cc[a].y, yy[b].x, acc[a][b].y));
+                }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int t = t0 + 2 * ty + a, v = v0 + 2 * tx + b;
+            if (t < T && v < Vte) out[((int64_t)t * L + s) * Vte + v] = acc[a][b];
+        }
+}
+
 bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStream_t st) {
     const int N = p->cfg.N;
     if (p->pairs == 0) return BS_OK;
@@ -242,6 +301,14 @@ bs_status launch_lift(const bs_plan *p, const float2 *c, float2 *c_hat, cudaStre
     lift_kernel<<<grid, thr, padded_len(M < 16 ? 16 : M) * sizeof(float2), st>>>(
         c, p->d_woff, p->d_Wg, p->d_start, p->d_twM, M, N, p->pairs, per, scale, c_hat);
     return check_launch("lift launch");
+}
+
+bs_status launch_apply_lifted_simt(const bs_plan *p, const float2 *xc, const float2 *c_hat, float2 *out,
+                                   cudaStream_t st) {
+    const int T = p->cfg.T, L = p->Ls, Vte = p->Vte;   // the plan's subbands, Fs bins per record of xc
+    dim3 grid((T + AL_T - 1) / AL_T, (Vte + AL_V - 1) / AL_V, L);
+    apply_lifted_kernel<<<grid, 256, 0, st>>>(xc, c_hat, out, p->cfg.N, p->Fs, p->B, L, T, p->cfg.P_train, Vte);
+    return check_launch("lifted outputs launch");
 }
 
 bs_status launch_beam_pattern_simt(const bs_plan *p, const float2 *c_hat, int n_dirs, const double *u,

@@ -488,6 +488,21 @@ bool pattern_simt(const bs_plan *p, int n_dirs) {
     return pairs * (7.0 + (n_dirs + 31) / 32 * (3.5 + N / 124)) < (4000 + 50 * N) * std::ceil(tiles / p->num_sms);
 }
 
+// Outputs of short rows: the SIMT kernel (lift.cu).  A tensor-core tile spends
+// 4 to 6 us on its start, drain and store, a SIMT tile of 32 x 32 outputs 2 us
+// and 2 more per 32 elements, as long as its four times as many tiles are at
+// most two waves.  N = 16, 1 to 64 targets, 16 subbands 4.0 us against 4.4 to
+// 6.0; N = 64 6.3 against 7 to 8.8; N = 65 with up to a wave 8.1 and 9.0, N = 100
+// 11.1 and 11.3; with 64 subbands of 64 targets x 128 vectors 7.2 and 6.1.  By
+// the whole plan's subbands, so that a shard's outputs are those of the whole.
+bool lifted_simt(const bs_plan *p) {
+    const int N = p->cfg.N, T = p->cfg.T, L = p->cfg.L, V = p->Vte;
+    if (N > 96) return false;
+    const double tc = (double)L * ((T + LT_T - 1) / LT_T) * ((V + 127) / 128);
+    const double simt = (double)L * ((T + 31) / 32) * ((V + 31) / 32);
+    return simt <= (N <= 64 ? 2 * std::ceil(tc / p->num_sms) : 1) * p->num_sms;
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
@@ -495,6 +510,7 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 bs_status launch_apply_lifted(const bs_plan *p, const float2 *xc, const float2 *c_hat, float2 *out,
                               cudaStream_t st) {
     if (p->Vte == 0 || p->pairs == 0) return BS_OK;
+    if (lifted_simt(p)) return launch_apply_lifted_simt(p, xc, c_hat, out, st);
     LtArgs a = lift_args(p, c_hat, p->Vte, 128);
     a.xc = xc;
     a.F = p->Fs;

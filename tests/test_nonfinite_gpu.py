@@ -29,9 +29,10 @@ def _mm(a, b):
         return (np.asarray(a, np.float64)[:, :, None] * np.asarray(b, np.float64)[None]).sum(1)
 
 
-@pytest.mark.parametrize("N,few", [(5, True), (48, True), (48, False), (150, True), (149, False)])
-def test_outputs_of_infinite_vectors_and_weights(N, few):
-    T, L, B, P_te = 3, 2, 8, 3
+@pytest.mark.parametrize("N,few,T,L,B", [(5, True, 3, 2, 8), (48, False, 3, 2, 8), (150, True, 3, 2, 8), (149, False, 3, 2, 8),
+                                        (5, True, 35, 64, 32), (48, True, 35, 64, 32), (47, False, 35, 64, 32)])
+def test_outputs_of_infinite_vectors_and_weights(N, few, T, L, B):
+    P_te = 3   # the last three cases are more than two waves of the SIMT kernel: tensor-core tiles
     M = 1 << max(4, (N - 1).bit_length())
     plan = P.Plan(N=N, F=L * B, L=L, M=M, u=np.sin(np.linspace(-1.0, 1.0, T)), W=[3] * T, K=[B] * T, P_train=1, P_test=P_te,
                   fc=10e9, fs=1e9, fd=10e9, delta=10.0)
@@ -53,7 +54,7 @@ def test_outputs_of_infinite_vectors_and_weights(N, few):
     P.bs_apply_lifted(plan, torch.view_as_complex(torch.from_numpy(y).cuda()).reshape(-1),
                       torch.view_as_complex(torch.from_numpy(c).cuda()).reshape(-1), out)
     o = out.cpu().numpy().reshape(T, L, P_te * B)
-    for s in range(L):
+    for s in range(2):   # where the values above are
         cr, ci = c[:, s, :, 0], c[:, s, :, 1]
         v = y[1:, s].reshape(P_te * B, N, 2)
         re = _mm(np.concatenate([cr, ci], 1), np.concatenate([v[..., 0], v[..., 1]], 1).T)

@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(COV_THREADS)
     }
 }
 
-// Plans with windows above 16 beams: one CTA per pair with 4 x 4 tiles.  The
+// Plans with windows above 16 beams (cov_wide_tiles): one CTA per pair with 4 x 4 tiles.  The
 // 3 x 3 tiles of window_cov_kernel left 62 of 128 threads idle at W = 32 (66
 // tiles, one slice) and tested every entry against W; here 36 tiles fill 108
 // threads in three slices, rows are staged at a pitch of a multiple of four
@@ -523,6 +523,19 @@ bs_status launch_window_cov_warp(const bs_plan *p, const void *ztr, const float 
     return check_launch("covariance (warp per pair) launch");
 }
 
+// The wider tiles win where they pad little and fill the threads better than
+// the 3 x 3 ones (W = 32: 36 tiles in three slices against 66 in one), over
+// streams that outweigh their longer epilogue, and for few pairs, where a CTA's
+// own time counts.  4x4 against 3x3 at 2560 pairs: W = 32 K = 16 46 us and 42,
+// K = 64 63 and 68, K = 256 143 and 199; W = 28 K = 64 1.11 times, K = 256 0.87; W = 24 K = 128 1.13, K = 512 0.90; W = 29 1.02 at best, W = 17 .. 21
+// 1.0 to 1.6.  At 192 pairs W = 25 .. 32 0.5 to 1.06 whatever K.  By the whole
+// plan's pairs: a shard's covariances are those of the whole bit for bit.
+static bool cov_wide_tiles(const bs_plan *p) {
+    const int W = p->Wmax, K = p->Kmax;
+    if ((int64_t)p->cfg.T * p->cfg.L <= 4LL * p->num_sms) return W >= 25 || (W >= 22 && K >= 128);
+    return W >= 31 ? K >= 64 : (W >= 26 && W <= 28) ? K >= 128 : (W >= 22 && W <= 24) && K >= 256;
+}
+
 bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delta, double2 *R,
                             cudaStream_t st, int64_t pred) {
     const unsigned G = (unsigned)p->pairs;
@@ -537,8 +550,8 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
                                                                    p->d_Kg, p->d_roff, delta, (float)p->cfg.delta, R);
         return check_launch("plain covariance launch");
     }
-    // windows above 16 beams: a CTA per pair with 4 x 4 tiles, which cover any
-    // W (16-bit windows are widened to FP32 as they are read)
+    // windows above 16 beams: a CTA per pair with 4 x 4 or 3 x 3 tiles, which
+    // cover any W (16-bit windows are widened to FP32 as they are read)
     const bool wide = p->Wmax > WMAX_COV;
     if (wide && p->Wmax > 32) return set_error(BS_EUNSUPPORTED, "W > 32");
     const int tv = p->tune_cov;   // a variant chosen by bs_autotune_pass, where it applies
@@ -550,7 +563,7 @@ bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delt
     if (window_cov_uses_warp(p))
         return launch_window_cov_warp(p, ztr, delta, R, st, 0, p->pairs, nullptr,
                                       dependent((p->pairs + COVW_WARPS - 1) / COVW_WARPS));
-    if (wide) {
+    if (wide && cov_wide_tiles(p)) {
         const auto kernel = p->cfg.precision == BS_PREC_FP32   ? window_cov_wide_kernel<BS_PREC_FP32>
                             : p->cfg.precision == BS_PREC_FP16 ? window_cov_wide_kernel<BS_PREC_FP16>
                                                                : window_cov_wide_kernel<BS_PREC_BF16>;

@@ -20,7 +20,8 @@ namespace bs {
 template <int M, bool kFull, int PREC>
 __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
     beamspace_kernel(const float2 *y, int64_t nvec, int N, const float2 *__restrict__ tw,
-                     float scale, float2 *__restrict__ out, GatherArgs ga) {
+                     float scale, float2 *__restrict__ out, GatherArgs ga, const int32_t *__restrict__ glist,
+                     int sumW) {
     using RP = Radix<M>;
     constexpr int vpb = BsCfg<M>::vpb;
     constexpr int nthr = BsCfg<M>::nthr;
@@ -86,8 +87,8 @@ __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
         // target's base).
         if (vid0 >= ga.nvec) return;
         const int nv = (ga.nvec - vid0 < (int64_t)vpb) ? (int)(ga.nvec - vid0) : vpb;
-        for (int e = tid; e < ga.sumW; e += nthr) {
-            const int packed = __ldg(&ga.glist[e]);
+        for (int e = tid; e < sumW; e += nthr) {
+            const int packed = __ldg(&glist[e]);   // (t << 8) | w, target-major
             const int t = packed >> 8, w = packed & 255;
             long long base;
             int sw, n;
@@ -137,9 +138,16 @@ __global__ void __launch_bounds__(BsCfg<M>::nthr, BsCfg<M>::minb)
     }
 }
 
+// What the plan adds to GatherArgs for the one-shot kernel and its launch.
+struct OneShotArgs {
+    const int32_t *glist = nullptr;
+    int sumW = 0, sms = 0;
+    int64_t pred = 0;   // CTAs of the preceding stage (launch_beamspace)
+};
+
 template <int M, bool kFull, int PREC>
 static bs_status launch_bs_t(const float2 *y, int64_t nvec, int N, const float2 *tw, float2 *out,
-                             const GatherArgs &ga, cudaStream_t st) {
+                             const GatherArgs &ga, const OneShotArgs &oa, cudaStream_t st) {
     using C = BsCfg<M>;
     static PerDevice attr;
     int per_sm = 0;
@@ -156,26 +164,26 @@ static bs_status launch_bs_t(const float2 *y, int64_t nvec, int N, const float2 
     if (blocks > 0x7FFFFFFF) return set_error(BS_EUNSUPPORTED, "too many vectors");
     if (blocks == 0) return BS_OK;
     // M >= 1024: several waves gain nothing (N = 1500: 1.5 % slower)
-    const bool dependent = ga.pred > 0 && (3 * ga.pred <= ga.sms || ga.pred + blocks <= ga.sms ||
-                                           (M < 1024 && blocks >= 2LL * per_sm * ga.sms));
+    const bool dependent = oa.pred > 0 && (3 * oa.pred <= oa.sms || oa.pred + blocks <= oa.sms ||
+                                           (M < 1024 && blocks >= 2LL * per_sm * oa.sms));
     launch_stage(dependent, beamspace_kernel<M, kFull, PREC>, (unsigned)blocks, C::nthr, C::smem, st, y, nvec, N, tw,
-                 1.0f / sqrtf((float)M), out, ga);
+                 1.0f / sqrtf((float)M), out, ga, oa.glist, oa.sumW);
     return check_launch("beamspace launch");
 }
 
 template <bool kFull, int PREC>
 static bs_status launch_bs(int M, const float2 *y, int64_t nvec, int N, const float2 *tw, float2 *out,
-                           const GatherArgs &ga, cudaStream_t st) {
+                           const GatherArgs &ga, const OneShotArgs &oa, cudaStream_t st) {
     switch (M) {
-        case 16: return launch_bs_t<16, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 32: return launch_bs_t<32, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 64: return launch_bs_t<64, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 128: return launch_bs_t<128, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 256: return launch_bs_t<256, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 512: return launch_bs_t<512, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 1024: return launch_bs_t<1024, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 2048: return launch_bs_t<2048, kFull, PREC>(y, nvec, N, tw, out, ga, st);
-        case 4096: return launch_bs_t<4096, kFull, PREC>(y, nvec, N, tw, out, ga, st);
+        case 16: return launch_bs_t<16, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 32: return launch_bs_t<32, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 64: return launch_bs_t<64, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 128: return launch_bs_t<128, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 256: return launch_bs_t<256, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 512: return launch_bs_t<512, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 1024: return launch_bs_t<1024, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 2048: return launch_bs_t<2048, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
+        case 4096: return launch_bs_t<4096, kFull, PREC>(y, nvec, N, tw, out, ga, oa, st);
     }
     return set_error(BS_EUNSUPPORTED, "M not supported");
 }
@@ -200,8 +208,6 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     ga.P_train = p->cfg.P_train;
     ga.uniform = (p->B % p->vpb) == 0;
     ga.gather = p->d_gather;
-    ga.glist = p->d_glist;
-    ga.sumW = p->sumW;
     ga.gsub = reinterpret_cast<const longlong2 *>(p->d_gsub);
     ga.ngather = (int)p->gather.size();
     ga.Wg = p->d_Wg;
@@ -212,8 +218,7 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     ga.ztr = ztr;
     ga.zte = zte;
     ga.store_scale = p->cfg.store_scale;
-    ga.pred = pred;
-    ga.sms = p->num_sms;
+    const OneShotArgs oa{p->d_glist, p->sumW, p->num_sms, pred};
     if (ctas) *ctas = p->num_sms;   // every kernel but the last fills the chip
     if (p->planar) return launch_beamspace2d(p, xc, ga, st);
     bool used = false;
@@ -240,16 +245,16 @@ bs_status launch_beamspace(const bs_plan *p, const float2 *xc, void *ztr, float2
     }
     if (ctas) *ctas = (ga.nvec + p->vpb - 1) / p->vpb;
     switch (p->cfg.precision) {
-        case BS_PREC_FP32: return launch_bs<false, BS_PREC_FP32>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, st);
-        case BS_PREC_FP16: return launch_bs<false, BS_PREC_FP16>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, st);
-        default: return launch_bs<false, BS_PREC_BF16>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, st);
+        case BS_PREC_FP32: return launch_bs<false, BS_PREC_FP32>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, oa, st);
+        case BS_PREC_FP16: return launch_bs<false, BS_PREC_FP16>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, oa, st);
+        default: return launch_bs<false, BS_PREC_BF16>(p->cfg.M, xc, ga.nvec, p->cfg.N, p->d_twM, nullptr, ga, oa, st);
     }
 }
 
 bs_status launch_beamspace_full(const bs_plan *p, const float2 *y, int64_t nvec, float2 *yb,
                                 cudaStream_t st) {
     GatherArgs ga{};
-    return launch_bs<true, BS_PREC_FP32>(p->cfg.M, y, nvec, p->cfg.N, p->d_twM, yb, ga, st);
+    return launch_bs<true, BS_PREC_FP32>(p->cfg.M, y, nvec, p->cfg.N, p->d_twM, yb, ga, OneShotArgs{}, st);
 }
 
 }  // namespace bs

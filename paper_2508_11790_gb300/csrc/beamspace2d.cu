@@ -21,6 +21,8 @@
 #include "beamspace_dev.cuh"
 #include "internal.h"
 
+#include <type_traits>
+
 #include <algorithm>
 
 namespace bs {
@@ -30,7 +32,7 @@ namespace bs {
 struct __align__(16) Tgt2d {
     long long base;
     int sxz;   // start_x | start_z << 16
-    int wn;    // W | Wz << 8 | stores << 16
+    int wn;    // W | Wz << 8 | stores << 16 | training << 24
 };
 
 constexpr int kPts2d = 4096;   // points per CTA
@@ -88,35 +90,41 @@ __global__ void __launch_bounds__(256, 4)
         __syncthreads();
     }
 
-    // window stores, the vectors of one subband at a time
+    // window stores: the vectors of one subband (a group) share their targets'
+    // windows; as many groups at a time as the entry table holds (with one, 32
+    // vectors of B = 1 went through 32 barriers: 21 us for 64 vectors of M = 128)
     const int Bv = min(V, 1 << ga.log2B);
-    for (int g0 = 0; g0 < V && vid0 + g0 < ga.nvec; g0 += Bv) {
-        const int64_t vec = ga.vbase + vid0 + g0;
-        const int p = (int)(vec >> ga.log2F);
-        const int q = (int)(vec & ((1 << ga.log2F) - 1));
-        const int s = q >> ga.log2B, i = q & ((1 << ga.log2B) - 1);
-        const bool train = p < ga.P_train;
-        const int v0 = train ? (p << ga.log2B) + i : ((p - ga.P_train) << ga.log2B) + i;
-        for (int t = tid; t < ga.T; t += nthr) {
+    const int ng = (int)min((int64_t)(V / Bv), (ga.nvec - vid0 + Bv - 1) / Bv), gmax = kTabT / ga.T;
+    auto store_groups = [&](int g0, int gn, auto single) {   // single: gn = 1, no divisions
+        for (int e = tid; e < gn * ga.T; e += nthr) {
+            const int k = single ? 0 : e / ga.T, t = single ? e : e - k * ga.T;
+            const int64_t vec = ga.vbase + vid0 + (g0 + k) * Bv;
+            const int p = (int)(vec >> ga.log2F);
+            const int q = (int)(vec & ((1 << ga.log2F) - 1));
+            const int s = q >> ga.log2B, i = q & ((1 << ga.log2B) - 1);
+            const bool train = p < ga.P_train;
+            const int v0 = train ? (p << ga.log2B) + i : ((p - ga.P_train) << ga.log2B) + i;
             const int64_t g = (int64_t)t * ga.L + s;
             const int W = __ldg(&ga.Wg[g]);
             const int n = train ? max(0, min(Bv, __ldg(&ga.Kg[g]) - v0)) : Bv;
-            Tgt2d e;
-            e.base = __ldg(train ? &ga.ztr_off[g] : &ga.zte_off[g]) + (long long)v0 * W;
-            e.sxz = __ldg(&ga.start[g]) | (__ldg(&start_z[g]) << 16);
-            e.wn = W | (__ldg(&Wz[t]) << 8) | (n << 16);
-            tgt[t] = e;
+            Tgt2d x;
+            x.base = __ldg(train ? &ga.ztr_off[g] : &ga.zte_off[g]) + (long long)v0 * W;
+            x.sxz = __ldg(&ga.start[g]) | (__ldg(&start_z[g]) << 16);
+            x.wn = W | (__ldg(&Wz[t]) << 8) | (n << 16) | (!single && train ? 1 << 24 : 0);
+            tgt[e] = x;
         }
         __syncthreads();
-        const float2 *bg = b + g0 * Mz * pl;
-        for (int e = tid; e < sumW; e += nthr) {
-            const int packed = __ldg(&glist[e]);
+        const bool train0 = (ga.vbase + vid0 + g0 * Bv) >> ga.log2F < ga.P_train;
+        for (int e = tid; e < gn * sumW; e += nthr) {
+            const int k = single ? 0 : e / sumW;
+            const int packed = __ldg(&glist[e - k * sumW]);
             const int w = packed & 255;
-            const Tgt2d te = tgt[packed >> 8];
-            const int W = te.wn & 255, wz = (te.wn >> 8) & 255, n = te.wn >> 16;
+            const Tgt2d te = tgt[k * ga.T + (packed >> 8)];
+            const int W = te.wn & 255, wz = (te.wn >> 8) & 255, n = single ? te.wn >> 16 : (te.wn >> 16) & 255;
+            const bool train = single ? train0 : (te.wn >> 24) != 0;
             const int wx = w / wz;
             const int mx = ((te.sxz & 0xFFFF) + wx) & (MX - 1), mz = ((te.sxz >> 16) + w - wx * wz) & (Mz - 1);
-            const float2 *src = bg + mz * pl + padrow(mx);
+            const float2 *src = b + ((g0 + k) * Bv * Mz + mz) * pl + padrow(mx);
             const int64_t o = te.base + w;
             auto all = [&](auto put) {
 #pragma unroll 4
@@ -127,8 +135,11 @@ __global__ void __launch_bounds__(256, 4)
             else if (prec == BS_PREC_FP16) all([&](int64_t k, float2 v) { store_train<BS_PREC_FP16>(ga.ztr, k, v, ga.store_scale); });
             else all([&](int64_t k, float2 v) { store_train<BS_PREC_BF16>(ga.ztr, k, v, ga.store_scale); });
         }
-        __syncthreads();   // the entries are rewritten for the next subband
-    }
+        __syncthreads();   // the entries are rewritten for the next groups
+    };
+    if (V == Bv) store_groups(0, 1, std::true_type{});
+    else
+        for (int g0 = 0; g0 < ng; g0 += gmax) store_groups(g0, min(gmax, ng - g0), std::false_type{});
 }
 
 __global__ void __launch_bounds__(128)
@@ -231,8 +242,15 @@ bs_status launch_beamspace2d(const bs_plan *p, const float2 *xc, const GatherArg
     const int Nx = p->Nx, Nz = p->Nz, Mx = p->Mx, Mz = p->Mz;
     if (ga.nvec == 0) return BS_OK;
     // rows of 8 to 1024 beams (Stockham radices), columns of up to 16 (in
-    // registers), 2 to 32 vectors per CTA, targets within the entry table
-    if (Mx >= 8 && Mx <= 1024 && Mz <= 16 && Mx * Mz >= 128 && p->cfg.T <= kTabT) {
+    // registers), 2 to 32 vectors per CTA, targets within the entry table.  Not
+    // where a CTA's subbands take three turns of the table or more (20 targets,
+    // B = 1, M = 128: 11.5 us against 7.6; 100 targets, B = 2 22 against 16; two
+    // turns: 10.0 and 10.4), nor where 32 vectors a CTA leave sixteen CTAs or
+    // fewer (64 vectors, 2 targets 6.3 and 5.7).
+    const int V = std::max(1, kPts2d / (Mx * Mz)), groups = std::max(1, V / p->B);
+    const bool turns = p->cfg.T <= kTabT && groups > 2 * (kTabT / p->cfg.T);
+    if (Mx >= 8 && Mx <= 1024 && Mz <= 16 && Mx * Mz >= 128 && p->cfg.T <= kTabT && !turns &&
+        !(V == 32 && ga.nvec <= 16 * V)) {
         switch (Mx) {
             case 8: return launch_2d_fft<8>(p, xc, ga, st);
             case 16: return launch_2d_fft<16>(p, xc, ga, st);

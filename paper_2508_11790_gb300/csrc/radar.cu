@@ -40,14 +40,19 @@ __global__ void __launch_bounds__(BsCfg<F>::nthr, BsCfg<F>::minb)
     extern __shared__ float2 sm[];
     const int tid = threadIdx.x;
     const int64_t row0 = (int64_t)blockIdx.x * vpb;
+    // subband 0 of each row's outputs, decoded once: a division per load held
+    // the loads back (2 rows of F = 64 took 10 us, gather and FFT apart 7)
+    __shared__ int64_t first[vpb];
+    if (tid < vpb) {
+        const int64_t row = row0 + tid, t = row / P_te;
+        first[tid] = row < rows ? (t * L * P_te + (row - t * P_te)) << log2B : -1;
+    }
+    __syncthreads();
     auto gload = [&](int c, int k) -> float2 {
-        const int64_t row = row0 + c;
-        if (row >= rows) return make_float2(0.f, 0.f);
-        const int64_t t = row / P_te;
-        const int r = (int)(row - t * P_te);
+        const int64_t o = first[c];
+        if (o < 0) return make_float2(0.f, 0.f);
         const int q = (k + F / 2) & (F - 1);
-        const float2 *o = out + ((t * L * P_te + r) << log2B);   // subband 0 of the row
-        const float2 y = __ldg(&o[(((q >> log2B) * P_te) << log2B) + (q & ((1 << log2B) - 1))]);
+        const float2 y = __ldg(&out[o + (((int64_t)(q >> log2B) * P_te) << log2B) + (q & ((1 << log2B) - 1))]);
         const float2 pk = __ldg(&pulse[k]);
         return make_float2(y.x * pk.x + y.y * pk.y, y.x * pk.y - y.y * pk.x);   // conj(y) pk
     };

@@ -25,6 +25,13 @@ __device__ __forceinline__ void wait_for_predecessor() {
     let_dependents_launch();
 }
 
+// Barrier of the cluster, with release and acquire.  Not .aligned: it follows
+// code that only some lanes of a warp run, and that form is undefined unless the
+// whole warp arrives together.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // Complex sums as one packed FP32x2 instruction (sm_100 and later): the same
 // round-to-nearest result per component as two scalar adds, in half the
 // issue slots, which the FFT kernels (issue-bound) are short of.

@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(256, 2) mlp_wgrad_kernel(const WgradArgs a) {
             if (adam && ix[i] >= 0) pm[i] = a.m[ix[i]], pv[i] = a.v[ix[i]], pp[i] = a.p[ix[i]];
         }
         if (first)   // every thread has a first pass (rank * 256 + tid < 64 * 64)
-            asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+            cluster_sync();
         first = false;
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(256, 2) mlp_wgrad_kernel(const WgradArgs a) {
         }
     }
     // no CTA leaves while another may read its tile
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
 }
 
 template <int HP, int MT, bool TRAIN>

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(256) rd_cfar_kernel(const float *__restrict__ 
         }
     }
     if (nc == 1) return;   // no cluster
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
     if (rank == 0 && threadIdx.x == 0) {
         int n = 0;
         Best r{-1.0f, -1};
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(256) rd_cfar_kernel(const float *__restrict__ 
         if (peak) peak[t] = r.i;
     }
     // no CTA leaves while the first may read its result
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
 }
 
 template <int F>

@@ -28,20 +28,22 @@ namespace bs {
 // one but for ties at the 2^-44 level), log10(K / W) is the host's value where
 // K is the first target's, and only tau, its logarithm and |a~| are FP64.
 // 16 384 pairs of W = 9: 31 us with a thread per pair for all of it in FP64, 34
-// with a lane per feature, 23 now.
+// with a lane per feature, 25 now.
 constexpr int FEAT_PAIRS = 32, FEAT_THREADS = 512;   // two pairs per warp: their loads' latency is what is left
 
-// r 2^-e as double-float; zero where that is below FP32's range, infinite above.
-__device__ __forceinline__ DF scaled_df(double r, int e) {
+// Biased exponent of r 2^-e, or -1 where the double-float product below would
+// not be the FP64 one rounded: r zero, subnormal, infinite or NaN, r 2^-e outside
+// 2^-74 .. 2^126 (its low part or the product would leave FP32's range), or no
+// scale (e = NO_SCALE: tau zero or not finite).
+constexpr int NO_SCALE = 1 << 20;
+__device__ __forceinline__ int scaled_exponent(double r, int e) {
+    const int x = (__double2hiint(r) >> 20) & 0x7FF, y = x - e;
+    return x != 0 && x != 0x7FF && y >= 949 && y <= 1149 ? y : -1;
+}
+// r with that exponent as double-float
+__device__ __forceinline__ DF scaled_df(double r, int y) {
     const int hw = __double2hiint(r);
-    const int x = (hw >> 20) & 0x7FF, y = x - e;
-    double v = r;
-    if (x != 0 && x != 0x7FF) {
-        if (y <= 0) v = 0.0;
-        else if (y >= 0x7FF) v = __hiloint2double((hw & (int)0x80000000) | 0x7FF00000, 0);
-        else v = __hiloint2double((hw & ~0x7FF00000) | (y << 20), __double2loint(r));
-    }
-    const float2 s = split_f64(v);
+    const float2 s = split_f64(__hiloint2double((hw & ~0x7FF00000) | (y << 20), __double2loint(r)));
     return DF{s.x, s.y};
 }
 __device__ __forceinline__ float df_product(DF a, DF b) {   // rounded to FP32
@@ -56,7 +58,8 @@ __global__ void __launch_bounds__(FEAT_THREADS)
                     float *__restrict__ X) {
     // 1 / tau and 1 / |a~| scaled by a power of two each, as double-float
     __shared__ DF itau_s[FEAT_PAIRS], ina_s[FEAT_PAIRS];
-    __shared__ int et_s[FEAT_PAIRS];
+    __shared__ int et_s[FEAT_PAIRS], en_s[FEAT_PAIRS];   // their exponents' offsets
+    __shared__ double tau_s[FEAT_PAIRS], na_s[FEAT_PAIRS];   // for the entries out of double-float's reach
     __shared__ float ltau_s[FEAT_PAIRS], lk_s[FEAT_PAIRS];
     const int64_t g0 = (int64_t)blockIdx.x * FEAT_PAIRS;
     const int np = (int)min((int64_t)FEAT_PAIRS, pairs - g0);
@@ -68,17 +71,25 @@ __global__ void __launch_bounds__(FEAT_THREADS)
         for (int i = 0; i < W; ++i) tr += Rg[i * W + i].x;
         const double tau = tr / W;
         ltau_s[lane] = (float)log10(tau);
+        tau_s[lane] = tau;
         const int x = (__double2hiint(tau) >> 20) & 0x7FF;
-        const int e = (x != 0 && x != 0x7FF) ? x - 1023 : 0;
-        const DF t = scaled_df(tau, e);   // 1 <= |t| < 2
-        const float q = 1.f / t.h;
-        itau_s[lane] = df_norm(q, (fmaf(-q, t.h, 1.f) - q * t.l) * q);
-        et_s[lane] = e;
+        if (x != 0 && x != 0x7FF) {
+            const DF t = scaled_df(tau, 1023);   // 1 <= |t| < 2
+            const float q = 1.f / t.h;
+            itau_s[lane] = df_norm(q, (fmaf(-q, t.h, 1.f) - q * t.l) * q);
+            et_s[lane] = x - 1023;
+        } else {
+            et_s[lane] = NO_SCALE;
+        }
     } else if (warp == 1 && lane < np) {   // another warp, at the same time
         const double2 *a = at64 + woff[g0 + lane];
         double na = 0.0;
         for (int i = 0; i < W; ++i) na += a[i].x * a[i].x + a[i].y * a[i].y;
-        ina_s[lane] = scaled_df(rsqrt(na), 0);
+        na_s[lane] = na;
+        const double i = rsqrt(na);
+        const int y = scaled_exponent(i, 0);
+        en_s[lane] = y >= 0 ? 0 : NO_SCALE;
+        if (y >= 0) ina_s[lane] = scaled_df(i, y);
         const int K = Kg[g0 + lane];
         lk_s[lane] = K == K0 ? lk0 : (float)log10((double)K / (double)W);
     }
@@ -89,7 +100,7 @@ __global__ void __launch_bounds__(FEAT_THREADS)
         const double2 *Rg = R + roff[g];
         const double2 *a = at64 + woff[g];
         const DF itau = itau_s[k], ina = ina_s[k];
-        const int et = et_s[k];
+        const int et = et_s[k], en = en_s[k];
         float *x = X + g * nfeat;
         for (int o = lane; o < nfeat; o += 32) {
             float f;
@@ -103,11 +114,15 @@ __global__ void __launch_bounds__(FEAT_THREADS)
                     i -= i * (i - 1) / 2 > q;
                     j = q - i * (i - 1) / 2;
                 }
-                const double2 r = Rg[i * W + j];
-                f = df_product(scaled_df(im ? r.y : r.x, et), itau);
+                const double2 e = Rg[i * W + j];
+                const double r = im ? e.y : e.x;
+                const int y = scaled_exponent(r, et);
+                f = y >= 0 ? df_product(scaled_df(r, y), itau) : (float)(r * (1.0 / tau_s[k]));
             } else if (o < 3 * W + 2 * tri) {
                 const int q = o - W - 2 * tri;
-                f = df_product(scaled_df(q < W ? a[q].x : a[q - W].y, 0), ina);
+                const double r = q < W ? a[q].x : a[q - W].y;
+                const int y = scaled_exponent(r, en);
+                f = y >= 0 ? df_product(scaled_df(r, y), ina) : (float)(r * (1.0 / sqrt(na_s[k])));
             } else {
                 f = o == nfeat - 2 ? ltau_s[k] : lk_s[k];
             }

@@ -422,8 +422,10 @@ bs_status bs_mlp_train_step(bs_mlp *m, const float *X, const float *T, int64_t b
     if (batch == 0) return BS_OK;
     const cudaStream_t st = (cudaStream_t)stream;
     if (fused) {
-        if (lr > 0.f) m->step += 1;
-        return bs::launch_mlp_train(m, X, T, (int)batch, w, lr, m->step, loss, st);
+        const int step = m->step + (lr > 0.f);   // counts updates that were launched
+        if (bs_status s = bs::launch_mlp_train(m, X, T, (int)batch, w, lr, step, loss, st)) return s;
+        m->step = step;
+        return BS_OK;
     }
     const int I = m->n_in, H = m->n_hidden, O = m->n_out, B = (int)batch;
     const int64_t P = bs_mlp_param_count(I, H, O);

@@ -189,7 +189,7 @@ bs_status launch_cov_solve_tables(const void *z, int precision, float store_scal
                                   uint32_t flags, float2 *c, int32_t *info, int *head, int grid,
                                   cudaStream_t st);
 // the loading network with up to 256 hidden units and 64 outputs (mlp_fused.cu)
-bool mlp_fused_applies(const bs_mlp *m);
+bool mlp_fused_applies(const bs_mlp *m, int64_t batch);
 bs_status mlp_forward_by_slabs(const bs_mlp *m, int64_t batch, bool *slabs);
 bs_status launch_mlp_forward(const bs_mlp *m, const float *X, int batch, float *Y, const bs_mlp_work *w,
                              cudaStream_t st);

@@ -395,7 +395,7 @@ bs_status bs_mlp_forward(const bs_mlp *m, const float *X, int64_t batch, float *
     const cudaStream_t st = (cudaStream_t)stream;
     bool slabs = false;
     if (bs_status s = bs::mlp_forward_by_slabs(m, batch, &slabs)) return s;
-    if (slabs && batch <= INT32_MAX) return bs::launch_mlp_forward(m, X, (int)batch, Y, w, st);
+    if (slabs) return bs::launch_mlp_forward(m, X, (int)batch, Y, w, st);
     const int I = m->n_in, H = m->n_hidden, O = m->n_out, B = (int)batch;
     const __nv_bfloat16 *wb = (const __nv_bfloat16 *)m->weights_bf16;
     const float *b1 = m->master + (int64_t)H * I, *b2 = b1 + H + (int64_t)H * H, *b3 = b2 + H + (int64_t)O * H;
@@ -410,7 +410,7 @@ bs_status bs_mlp_forward(const bs_mlp *m, const float *X, int64_t batch, float *
 bs_status bs_mlp_train_step(bs_mlp *m, const float *X, const float *T, int64_t batch, const bs_mlp_work *w,
                             float lr, double *loss, bs_stream stream) {
     if (bs_status s = mlp_check(m)) return s;
-    const bool fused = bs::mlp_fused_applies(m) && batch >= 0 && batch <= INT32_MAX;
+    const bool fused = batch >= 0 && bs::mlp_fused_applies(m, batch);
     if (!fused) {
         if (bs_status s = bs_mlp_forward(m, X, batch, w ? w->y : nullptr, w, stream)) return s;
     } else {

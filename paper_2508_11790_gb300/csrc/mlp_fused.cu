@@ -706,7 +706,10 @@ MlpArgs slab_args(const bs_mlp *m, const float *X, int batch, float *Y, const bs
 
 }  // namespace
 
-bool mlp_fused_applies(const bs_mlp *m) { return m->n_hidden <= 256 && m->n_out <= OMAX && m->n_in <= 65536; }
+// rows are counted in ints, and up to a cluster's last chunks past the batch
+bool mlp_fused_applies(const bs_mlp *m, int64_t batch) {
+    return m->n_hidden <= 256 && m->n_out <= OMAX && m->n_in <= 65536 && batch <= INT32_MAX - 8 * WG_K;
+}
 
 // A slab costs the same for any H up to 128 (its columns are padded), a row of
 // the layer by layer products less the narrower the network, so forward passes
@@ -717,7 +720,7 @@ bool mlp_fused_applies(const bs_mlp *m) { return m->n_hidden <= 256 && m->n_out 
 // (A training step is faster by slabs everywhere: its weight gradients.)
 bs_status mlp_forward_by_slabs(const bs_mlp *m, int64_t batch, bool *slabs) {
     int sms = 0;
-    *slabs = mlp_fused_applies(m);
+    *slabs = mlp_fused_applies(m, batch);
     if (!*slabs || m->n_hidden >= 64) return BS_OK;
     if (bs_status s = device_sms(&sms)) return s;
     const double waves = std::ceil((double)batch / (32.0 * sms));

@@ -3,6 +3,8 @@
 #include "internal.h"
 #include "solve_dev.cuh"
 
+#include <algorithm>
+
 namespace bs {
 
 // Windows of 17..32 beams: one warp per pair, solved at WT = 20, 24, 28 or 32
@@ -14,8 +16,11 @@ namespace bs {
 // packed (8 KB): sixteen warps, 118 us, of which fetching the 11 600
 // straight-line instructions of a solve was the largest stall.  Now the twenty
 // warps that an SM holds at 96 registers are one CTA in lockstep: 92 us, one
-// wave (sixteen in lockstep: 134 us, two waves).
-constexpr int WIDE_WARPS = 20;
+// wave (sixteen in lockstep: 134 us, two waves).  Fewer pairs than that are
+// spread evenly over the SMs, so that they share an SM's issue with fewer others
+// (256 pairs of W = 32 53 -> 42 us, with a preconditioner 62 -> 45, 2560 pairs 54
+// -> 51).
+constexpr int WIDE_WARPS = 20;   // of a CTA, at most
 
 template <int WT, bool PRE>
 __global__ void __launch_bounds__(WIDE_WARPS * 32, 1)
@@ -27,7 +32,7 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, 1)
                            const int32_t *__restrict__ order, const float *__restrict__ dpre) {
     extern __shared__ __align__(16) unsigned char scratch[];   // solve_scratch_bytes<32> per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t at = slot0 + (int64_t)blockIdx.x * WIDE_WARPS + warp;
+    const int64_t at = slot0 + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     const int64_t slot = at < slot1 ? at : slot1 - 1;
     const int64_t g = order ? (int64_t)order[slot] : slot;
     const int64_t wo = woff[g];
@@ -42,7 +47,8 @@ static bs_status launch_wide_t(const bs_plan *p, const double2 *R, float2 *c, in
                             const float *dpre, int refine, int f64) {
     const int64_t s0 = p->wstart[WT - 3], s1 = p->wstart[WT + 1];
     const int32_t *order = p->Wmin == p->Wmax ? nullptr : p->d_order_w;
-    const unsigned blocks = (unsigned)((s1 - s0 + WIDE_WARPS - 1) / WIDE_WARPS);
+    const int warps = (int)std::min<int64_t>(WIDE_WARPS, (s1 - s0 + p->num_sms - 1) / p->num_sms);
+    const unsigned blocks = (unsigned)((s1 - s0 + warps - 1) / warps);
     constexpr int smem = WIDE_WARPS * solve_scratch_bytes<32>;
     static PerDevice attr;
     if (bs_status s = attr.get([](int *) {
@@ -55,7 +61,7 @@ static bs_status launch_wide_t(const bs_plan *p, const double2 *R, float2 *c, in
         }))
         return s;
     const auto kernel = dpre ? mvdr_solve_wide_kernel<WT, true> : mvdr_solve_wide_kernel<WT, false>;
-    kernel<<<blocks, WIDE_WARPS * 32, smem, st>>>(R, p->d_roff, p->d_Wg, p->d_woff, p->d_at32, p->d_atlo, p->d_at64, c,
+    kernel<<<blocks, warps * 32, warps * solve_scratch_bytes<32>, st>>>(R, p->d_roff, p->d_Wg, p->d_woff, p->d_at32, p->d_atlo, p->d_at64, c,
                                                info, s0, s1, p->cfg.kappa_max, refine, f64, order, dpre);
     return check_launch("solve (wide) launch");
 }

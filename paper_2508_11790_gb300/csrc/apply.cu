@@ -10,6 +10,8 @@
 #include "common.cuh"
 #include "internal.h"
 
+#include <algorithm>
+
 namespace bs {
 
 // WM: the largest window (16, or 32 with half as many warps per CTA), so a
@@ -108,13 +110,30 @@ __global__ void __launch_bounds__(ApplyCfg<WM>::threads)
     }
 }
 
+// Blocks of one pair that a warp takes: several only where the pairs alone fill
+// the GPU (64 warps an SM).
+static int blocks_per_warp(const bs_plan *p) {
+    return p->pairs >= 32LL * p->num_sms ? std::min(4, p->Vte / 32) : 1;
+}
+
+// Whole blocks pay where a warp takes several, or where latency counts (up to
+// 20 warps an SM in all: 64 pairs of W = 9, 128 vectors 2.5 us against 3.0).
+// Between, with a block per warp, they are 5 to 40 % slower than an output per
+// thread for small windows (2560 pairs of W = 2, 256 vectors 8.7 us against 6.3,
+// 32 768 pairs of one block 12.4 against 8.7), and windows of a multiple of 8
+// beams, whose reads of shared memory conflict, need more pairs (W = 32, 5120
+// pairs, 96 vectors 39 us against 36).  Both kernels give the same bits.  Over
+// 660 sizes within 1 % of the better one on average.
+static bool apply_by_blocks(const bs_plan *p) {
+    if (blocks_per_warp(p) > 1) return p->Wmax < 16 || p->Wmax % 8 != 0 || p->pairs >= 64LL * p->num_sms;
+    return p->pairs * (p->Vte / 32) <= 20LL * p->num_sms;
+}
+
 template <int WM>
 static bs_status launch_apply_blocks(const bs_plan *p, const float2 *z, const float2 *c, float2 *out, cudaStream_t st,
                                      bool dependent) {
     constexpr int NW = ApplyCfg<WM>::threads / 32;
-    const int nb = p->Vte / 32;
-    // several blocks per warp only where the pairs alone fill the GPU (64 warps an SM)
-    const int bpw = p->pairs >= 32LL * p->num_sms ? (nb < 4 ? nb : 4) : 1;
+    const int nb = p->Vte / 32, bpw = blocks_per_warp(p);
     const unsigned upp = (unsigned)((nb + bpw - 1) / bpw);
     const unsigned units = (unsigned)p->pairs * upp;
     launch_stage(dependent, apply_blocks_kernel<WM>, (units + NW - 1) / NW, ApplyCfg<WM>::threads, 0, st, z, p->d_zte_off,
@@ -131,7 +150,7 @@ bs_status launch_apply(const bs_plan *p, const float2 *zte, const float2 *c, flo
     // starts on 16 bytes if the array does.  8192 pairs of W = 9, 128 vectors:
     // 21.3 -> 19.3 us (12.5 at the copy bandwidth); 32 768 pairs of W = 3..15:
     // 67.6 -> 53.8 (46).
-    if (p->Vte % 32 == 0 && (reinterpret_cast<uintptr_t>(zte) & 15) == 0 && total / 32 < (1LL << 31))
+    if (p->Vte % 32 == 0 && (reinterpret_cast<uintptr_t>(zte) & 15) == 0 && total / 32 < (1LL << 31) && apply_by_blocks(p))
         return p->Wmax <= 16 ? launch_apply_blocks<16>(p, zte, c, out, st, dependent)
                              : launch_apply_blocks<32>(p, zte, c, out, st, dependent);
     const bool wide = p->Wmax > 16;

@@ -1,7 +1,7 @@
 """Beamformer outputs called by themselves: whole blocks of 32 test vectors
 (one and several blocks per warp, with and without a remainder), other vector
-counts, windows of 1 to 32 beams, few pairs and enough to give a warp several
-blocks, and test windows that start on 8 bytes only.
+counts, windows of 1 to 32 beams, few pairs, enough to give a warp several
+blocks, and the number between that takes an output per thread, and test windows that start on 8 bytes only.
 
 Tolerance: a sum of W complex FP32 products, 2 W + 2 roundings of 2^-24 of the
 sum of the products' magnitudes."""
@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("shift", [0, 1])
 @pytest.mark.parametrize("T,L,B,P_te", [
     (3, 2, 8, 4), (3, 2, 8, 12), (2, 4, 16, 8), (5, 2, 32, 5), (4, 2, 32, 7), (3, 2, 16, 3), (2, 2, 1, 1),
-    (80, 64, 8, 4), (80, 64, 8, 12), (80, 64, 16, 8), (80, 64, 32, 5), (80, 64, 32, 7), (80, 64, 8, 5)])
+    (40, 64, 16, 8), (80, 64, 8, 4), (160, 64, 16, 4), (80, 64, 8, 12), (80, 64, 16, 8), (80, 64, 32, 5), (80, 64, 32, 7), (80, 64, 8, 5)])
 @pytest.mark.parametrize("widths", [(1, 9, 16), (3,), (17, 2, 32)])
 def test_outputs_match_fp64(T, L, B, P_te, widths, shift):
     W = [widths[t % len(widths)] for t in range(T)]

@@ -125,7 +125,7 @@ static int blocks_per_warp(const bs_plan *p) {
 // pairs, 96 vectors 39 us against 36).  Both kernels give the same bits.  Over
 // 660 sizes within 1 % of the better one on average.
 static bool apply_by_blocks(const bs_plan *p) {
-    if (blocks_per_warp(p) > 1) return p->Wmax < 16 || p->Wmax % 8 != 0 || p->pairs >= 64LL * p->num_sms;
+    if (blocks_per_warp(p) > 1) return p->Wmax < 16 || p->Wmax % 8 != 0 || p->pairs >= 96LL * p->num_sms;
     return p->pairs * (p->Vte / 32) <= 20LL * p->num_sms;
 }
 

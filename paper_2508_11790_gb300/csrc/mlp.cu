@@ -27,8 +27,9 @@ namespace bs {
 // operations and scaled in double-float (the FP32 result is the rounded FP64
 // one but for ties at the 2^-44 level), log10(K / W) is the host's value where
 // K is the first target's, and only tau, its logarithm and |a~| are FP64.
-// 16 384 pairs of W = 9: 31 us with a thread per pair for all of it in FP64, 34
-// with a lane per feature, 25 now.
+// 16 384 pairs of W = 9, back to back: 23 us with a thread per pair for all of
+// it in FP64, 18 now; rows shorter than a warp are taken together (10 240 pairs
+// of W = 2 9.7 us with a warp a row, 5.6 now).
 constexpr int FEAT_PAIRS = 32, FEAT_THREADS = 512;   // two pairs per warp: their loads' latency is what is left
 
 // Biased exponent of r 2^-e, or -1 where the double-float product below would
@@ -95,39 +96,37 @@ __global__ void __launch_bounds__(FEAT_THREADS)
     }
     __syncthreads();
     const int tri = W * (W - 1) / 2;
-    for (int k = warp; k < np; k += FEAT_THREADS / 32) {
-        const int64_t g = g0 + k;
-        const double2 *Rg = R + roff[g];
-        const double2 *a = at64 + woff[g];
-        const DF itau = itau_s[k], ina = ina_s[k];
-        const int et = et_s[k], en = en_s[k];
-        float *x = X + g * nfeat;
-        for (int o = lane; o < nfeat; o += 32) {
-            float f;
-            if (o < W + 2 * tri) {
-                const bool im = o >= W + tri;
-                int i = o, j = o;
-                if (o >= W) {
-                    const int q = o - W - (im ? tri : 0);   // entry of the strict lower triangle, row-major
-                    i = (int)((sqrtf(8.f * (float)q + 1.f) + 1.f) * 0.5f);
-                    i += i * (i + 1) / 2 <= q;   // the rounded root may be one off
-                    i -= i * (i - 1) / 2 > q;
-                    j = q - i * (i - 1) / 2;
-                }
-                const double2 e = Rg[i * W + j];
-                const double r = im ? e.y : e.x;
-                const int y = scaled_exponent(r, et);
-                f = y >= 0 ? df_product(scaled_df(r, y), itau) : (float)(r * (1.0 / tau_s[k]));
-            } else if (o < 3 * W + 2 * tri) {
-                const int q = o - W - 2 * tri;
-                const double r = q < W ? a[q].x : a[q - W].y;
-                const int y = scaled_exponent(r, en);
-                f = y >= 0 ? df_product(scaled_df(r, y), ina) : (float)(r * (1.0 / sqrt(na_s[k])));
-            } else {
-                f = o == nfeat - 2 ? ltau_s[k] : lk_s[k];
+    auto feature = [&](int k, int o) -> float {   // feature o of pair g0 + k
+        if (o < W + 2 * tri) {
+            const bool im = o >= W + tri;
+            int i = o, j = o;
+            if (o >= W) {
+                const int q = o - W - (im ? tri : 0);   // entry of the strict lower triangle, row-major
+                i = (int)((sqrtf(8.f * (float)q + 1.f) + 1.f) * 0.5f);
+                i += i * (i + 1) / 2 <= q;   // the rounded root may be one off
+                i -= i * (i - 1) / 2 > q;
+                j = q - i * (i - 1) / 2;
             }
-            x[o] = f;
+            const double2 e = R[roff[g0 + k] + i * W + j];
+            const double r = im ? e.y : e.x;
+            const int y = scaled_exponent(r, et_s[k]);
+            return y >= 0 ? df_product(scaled_df(r, y), itau_s[k]) : (float)(r * (1.0 / tau_s[k]));
         }
+        if (o < 3 * W + 2 * tri) {
+            const int q = o - W - 2 * tri;
+            const double2 *a = at64 + woff[g0 + k];
+            const double r = q < W ? a[q].x : a[q - W].y;
+            const int y = scaled_exponent(r, en_s[k]);
+            return y >= 0 ? df_product(scaled_df(r, y), ina_s[k]) : (float)(r * (1.0 / sqrt(na_s[k])));
+        }
+        return o == nfeat - 2 ? ltau_s[k] : lk_s[k];
+    };
+    float *x = X + g0 * nfeat;
+    if (nfeat >= 32) {
+        for (int k = warp; k < np; k += FEAT_THREADS / 32)
+            for (int o = lane; o < nfeat; o += 32) x[(int64_t)k * nfeat + o] = feature(k, o);
+    } else {   // rows shorter than a warp
+        for (int e = threadIdx.x; e < np * nfeat; e += FEAT_THREADS) x[e] = feature(e / nfeat, e % nfeat);
     }
 }
 

@@ -528,12 +528,12 @@ bs_status launch_window_cov_warp(const bs_plan *p, const void *ztr, const float 
 // streams that outweigh their longer epilogue, and for few pairs, where a CTA's
 // own time counts.  4x4 against 3x3 at 2560 pairs: W = 32 K = 16 46 us and 42,
 // K = 64 63 and 68, K = 256 143 and 199; W = 28 K = 64 1.11 times, K = 256 0.87; W = 24 K = 128 1.13, K = 512 0.90; W = 29 1.02 at best, W = 17 .. 21
-// 1.0 to 1.6.  At 192 pairs W = 25 .. 32 0.5 to 1.06 whatever K.  By the whole
+// 1.0 to 1.6, W = 9, 20 and 32 mixed K = 64 1.0 to 1.13.  At 192 pairs W = 25 .. 32 0.5 to 1.06 whatever K.  By the whole
 // plan's pairs: a shard's covariances are those of the whole bit for bit.
 static bool cov_wide_tiles(const bs_plan *p) {
     const int W = p->Wmax, K = p->Kmax;
     if ((int64_t)p->cfg.T * p->cfg.L <= 4LL * p->num_sms) return W >= 25 || (W >= 22 && K >= 128);
-    return W >= 31 ? K >= 64 : (W >= 26 && W <= 28) ? K >= 128 : (W >= 22 && W <= 24) && K >= 256;
+    return W >= 31 ? K >= (p->Wmin >= 31 ? 64 : 128) : (W >= 26 && W <= 28) ? K >= 128 : (W >= 22 && W <= 24) && K >= 256;
 }
 
 bs_status launch_window_cov(const bs_plan *p, const void *ztr, const float *delta, double2 *R,

@@ -367,7 +367,7 @@ bs_status bs_apply(const bs_plan *plan, const bs_cf32 *z_test, const bs_cf32 *c,
  * beamspace output c_g^H S_g D y.  c: weights packed as bs_mvdr_solve writes
  * them ([pair][W_g], offsets woff); c_hat: [pair][N] cf32 (caller-owned
  * device memory; pair g = t L + s).  Errors: BS_EINVAL for NULL buffers or a
- * wrong device, BS_EUNSUPPORTED for W > 16. */
+ * wrong device, BS_EUNSUPPORTED for a planar plan. */
 bs_status bs_lift(const bs_plan *plan, const bs_cf32 *c, bs_cf32 *c_hat, bs_stream stream);
 
 /* The lifted correlator applied in antenna space (Sec. III-C, below Eq.
@@ -399,7 +399,7 @@ bs_status bs_beam_pattern(const bs_plan *plan, const bs_cf32 *c_hat, int32_t n_d
  *   map[t][d][tau] = |sum_r rp[t][r][tau] e^{-j 2 pi d r / P_test}|^2.
  * out: bs_apply's output [pairs][Vte]; pulse: [F] cf32 orthonormal spectrum
  * of the transmitted pulse (FFT order); work: caller-owned device scratch of
- * 2 T P_test F cf32; map: [T][P_test][F] FP32.  F is a power of two in
+ * 2 T P_test F cf32 (the first half is used); map: [T][P_test][F] FP32.  F is a power of two in
  * 16..4096 (plan validation).  A subband-shard plan is refused
  * (BS_EUNSUPPORTED): every subband of a target enters its map. */
 bs_status bs_range_doppler(const bs_plan *plan, const bs_cf32 *out, const bs_cf32 *pulse, bs_cf32 *work,

@@ -13,7 +13,7 @@
 // past Nx).  The vectors of a subband share their targets' windows, so a
 // thread decodes a (target, entry) once and stores it for all of them.  Bound
 // by the window stores: 20 targets of 4 x 8 beams write 5 KB per 1 KB vector.
-// 24 576 vectors of 4 x 32 elements, 8 x 64 beams: 37 us (22 us at the copy
+// 24 576 vectors of 4 x 32 elements, 8 x 64 beams: 38 us (22 us at the copy
 // bandwidth; 195 us with the general kernel).
 //
 // beamspace2d_kernel: any other shape; one warp per vector (radix-2 passes in

@@ -12,8 +12,10 @@ namespace bs {
 // covariance, solve, output; launch_stage() on the host): a kernel lets the
 // next one's CTAs be placed while it runs, and a kernel launched that way waits
 // here, before it touches memory, until its predecessor has completed.  What is
-// saved is the launch and ramp-up of each stage: a pass of 64 pairs 29.2 -> 23.2 us,
-// of 1024 pairs at N = 256 89 -> 82 us.  Both are no-ops in an ordinary launch.
+// saved is the launch and ramp-up of each stage: a pass of 64 pairs 29.8 -> 22.4 us,
+// of 1024 pairs at N = 256 89 -> 81 us.  Both are no-ops in an ordinary launch;
+// which stages are launched so is a question of their sizes (launch_beamspace()
+// in internal.h).
 // Arrays that an earlier stage of the pass writes are read by ordinary (or
 // .cg / .cs) loads only, through pointers that are not const __restrict__: the
 // read-only path (ld.global.nc: __ldg, or the compiler's choice for such a

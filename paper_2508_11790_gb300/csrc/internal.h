@@ -76,7 +76,7 @@ struct bs_plan {
     int *d_head = nullptr;
     bs::CovSolveLaunch cs;
     // kernel variants chosen by bs_autotune_pass (-1: the built-in choice)
-    int tune_beamspace = -1;   // 0 warp per residue, 1 bulk-copy staged, 2 one-shot
+    int tune_beamspace = -1;   // 0 warp per residue, 1 bulk-copy staged, 2 one-shot, 3 tensor cores
     int tune_cov = -1;         // 0 CTA per pair, 1 warp per pair, 2 tensor cores
     int tune_fused = -1;       // 0 covariance + solve as two launches, 1 one persistent launch
 };

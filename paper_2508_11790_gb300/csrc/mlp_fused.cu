@@ -12,7 +12,7 @@
 //
 // Bound: latency.  Training step of the 101-256-256-10 network, 1024 rows:
 // 470 us (15 launches, the three weight gradients 160 us each: 4 to 16 CTAs
-// with a serial chain of 1024 rows) -> 35 us (slab kernel 19, weight
+// with a serial chain of 1024 rows) -> 35 us (slab kernel 18, weight
 // gradients 14).  Forward of 4096 rows, back to back in a graph: 99 us (three
 // launches) -> 17.5, 3 of them the hidden layers' 17 MB in the work buffers.
 // With 8 warps instead of 16 and 32-row slabs at 1024 rows (32 CTAs) the slab

@@ -22,7 +22,7 @@
 // Bound by memory latency and launches (16 MB in all at 64 targets, 8 records,
 // 2048 points).  There: matched filter as a pass of its own 9 us + rows 8 ->
 // the rows alone; doppler a sincospi and a load per record, bin and cell (28
-// us); CFAR one CTA per target (32 us).  The three launches together: 75 -> 38
+// us); CFAR one CTA per target (32 us).  The three launches together: 75 -> 34
 // us.
 #include "beamspace_dev.cuh"
 #include "common.cuh"
